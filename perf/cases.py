@@ -165,6 +165,24 @@ def run(state):
     return out
 
 
+def exact(case, seed):
+    """The rounding study's log-plan by Algorithm 1 in its printed log-domain form, in fp64.  The masks
+    are picks, not computed numbers, and what they retain follows them."""
+    if case["kind"] != "ablation":
+        return None
+    m, M, N = prepare(case, seed)["mats"][0], case["M"], case["N"]
+    tau = torch.tensor(m.tau, dtype=torch.float32).double().item()     # the interface takes tau in fp32
+    x = m.w.double().abs_().mul_(tau).view(m.rows // M, M, m.cols // M, M).transpose(1, 2)
+    x, q = x.contiguous(), torch.zeros((), dtype=torch.float64, device="cuda")
+    for _ in range(case["iters"]):
+        x = x - torch.logsumexp(x, -1, keepdim=True) + math.log(N)
+        x = x - torch.logsumexp(x, -2, keepdim=True) + math.log(N)
+        y = x + q
+        x = y.clamp(max=0.0)
+        q = y - x
+    return [x.transpose(1, 2).reshape(m.rows, m.cols)] + [None] * 6
+
+
 def work(case):
     """Scores read once per call that needs them, masks (and the study's plan) written once; four
     fp32 operations per entry and iteration: clip, row sum, column sum, scaling.  The operations of
