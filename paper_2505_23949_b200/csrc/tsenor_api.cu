@@ -72,14 +72,14 @@ int make_source(const tsenor_scores_t* d, int64_t cols, tsenor::ScoreSrc* out) {
 
 std::atomic<int> g_layout{TSENOR_LAYOUT_AUTO};
 
-// Panels (= CTAs) a matrix is cut into under layout V.
+// Units (= warps) a matrix is cut into under layout V, and the slots of a block row: whole mask
+// words, except that a single block column needs no padding.
 template <int M, int V>
-int64_t panel_count(const tsenor::Params& P, bool tall, int64_t* npc_out) {
+int64_t unit_count(const tsenor::Params& P, int64_t* nbp_out) {
     using G = tsenor::Geom<M, V>;
-    constexpr int NB = G::PANEL / M;
-    const int64_t npc = (P.cols + G::PANEL - 1) / G::PANEL;
-    *npc_out = npc;
-    return tall ? (P.rows / M + NB - 1) / NB : (P.rows / M) * npc;
+    const int64_t nbc = P.cols / M, nbp = (nbc == 1) ? 1 : (nbc + G::GPW - 1) / G::GPW * G::GPW;
+    *nbp_out = nbp;
+    return ((P.rows / M) * nbp + G::BPW - 1) / G::BPW;
 }
 
 int sm_count() {
@@ -94,22 +94,20 @@ int sm_count() {
     return cached;
 }
 
-template <int M, int MODE, int V>
-int launch_layout(const tsenor::Params& P, bool tall, cudaStream_t st) {
+template <int M, int MODE, int V, bool EE>
+int launch_layout(const tsenor::Params& P, cudaStream_t st) {
     using G = tsenor::Geom<M, V>;
-    int64_t npc = 0;
-    const int64_t panels = panel_count<M, V>(P, tall, &npc);
-    if (panels == 0) return TSENOR_OK;
-    if (panels > 0x7fffffffLL) return TSENOR_ERR_SHAPE;
     tsenor::Params Q = P;
-    Q.npc = (int)npc;
-    Q.tall = tall ? 1 : 0;
-    const size_t smem = sizeof(tsenor::SmemLayout<G, MODE>);
+    const int64_t units = unit_count<M, V>(P, &Q.nbp);
+    if (units == 0) return TSENOR_OK;
+    if (units > 0x7fffffffLL) return TSENOR_ERR_SHAPE;
+    constexpr int WPC = tsenor::CtaWarps<M, V, EE>::value;
+    const size_t smem = WPC * sizeof(tsenor::SmemLayout<G, MODE, EE>);
     static thread_local int configured_device = -1;
     int dev = 0;
     cudaGetDevice(&dev);
     if (configured_device != dev) {
-        cudaError_t e = cudaFuncSetAttribute(tsenor::tsenor_kernel<M, MODE, V>,
+        cudaError_t e = cudaFuncSetAttribute(tsenor::tsenor_kernel<M, MODE, V, EE>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) {
             g_last_cuda_error = (int)e;
@@ -117,37 +115,43 @@ int launch_layout(const tsenor::Params& P, bool tall, cudaStream_t st) {
         }
         configured_device = dev;
     }
-    tsenor::tsenor_kernel<M, MODE, V><<<(unsigned)panels, tsenor::WARPS * 32, smem, st>>>(Q);
+    tsenor::tsenor_kernel<M, MODE, V, EE><<<(unsigned)((units + WPC - 1) / WPC), 32 * WPC, smem, st>>>(Q);
     return finish_launch();
 }
 
 // Chooses the register layout: the latency layout (a block over M lanes) when even its
-// finer panels leave the GPU with no more than four CTAs per SM, i.e. when the run time is
+// finer units leave the GPU with no more than 16 warps per SM, i.e. when the run time is
 // the chain of dependent iterations of a single warp rather than instruction throughput.
-template <int M, int MODE>
+template <int M, int MODE, bool EE>
 int launch(const tsenor::Params& P, cudaStream_t st) {
-    // a slab (single block column) is cut into panels of vertically stacked blocks
-    const bool tall = (P.cols == M) && (P.rows > M);
     if constexpr (M < 32) {   // a 32 x 32 block takes a whole warp in either layout
         const int policy = g_layout.load(std::memory_order_relaxed);
         bool fine = (policy == TSENOR_LAYOUT_LATENCY);
         if (policy == TSENOR_LAYOUT_AUTO) {
-            int64_t npc = 0;
-            fine = panel_count<M, 1>(P, tall, &npc) <= 4LL * sm_count();
+            int64_t nbp = 0;
+            fine = unit_count<M, 1>(P, &nbp) <= 16LL * sm_count();
         }
-        if (fine) return launch_layout<M, MODE, 1>(P, tall, st);
+        if (fine) return launch_layout<M, MODE, 1, EE>(P, st);
     }
-    return launch_layout<M, MODE, 0>(P, tall, st);
+    return launch_layout<M, MODE, 0, EE>(P, st);
 }
 
+template <int MODE, bool EE>
+int dispatch_size(const tsenor::Params& P, int M, cudaStream_t st) {
+    switch (M) {
+        case 4: return launch<4, MODE, EE>(P, st);
+        case 8: return launch<8, MODE, EE>(P, st);
+        case 16: return launch<16, MODE, EE>(P, st);
+        default: return launch<32, MODE, EE>(P, st);
+    }
+}
+
+// The stopping-test mode has kernels of its own: the test's code stays out of the others.
 template <int MODE>
 int dispatch(const tsenor::Params& P, int M, cudaStream_t st) {
-    switch (M) {
-        case 4: return launch<4, MODE>(P, st);
-        case 8: return launch<8, MODE>(P, st);
-        case 16: return launch<16, MODE>(P, st);
-        default: return launch<32, MODE>(P, st);
-    }
+    if constexpr (MODE != 2)
+        if (P.ee_eps > 0.0f && P.iters > 0) return dispatch_size<MODE, true>(P, M, st);
+    return dispatch_size<MODE, false>(P, M, st);
 }
 
 void set_tau(tsenor::Params& P, float tau) {
@@ -475,6 +479,7 @@ static int dykstra_on(const tsenor::ScoreSrc& src, const Extras& x, int64_t rows
     tsenor::Params P{};
     P.src = src;
     P.plan = plan_out; P.ld_plan = ld_plan; P.plan_is_log = plan_is_log;
+    P.vec_plan = aligned16(plan_out, ld_plan);
     P.rows = rows; P.cols = cols;
     P.N = N; P.Nf = (float)N; P.log2N = (float)std::log2((double)N);
     set_tau(P, tau);

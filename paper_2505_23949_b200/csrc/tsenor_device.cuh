@@ -2,19 +2,21 @@
 // Dykstra iterations (Algorithm 1), greedy selection and local search
 // (Algorithm 2, Eq. 6), bit-packed mask writer.
 //
-// Layout in one sentence: a CTA owns a panel of M rows x PANEL columns of the
-// score matrix (PANEL = WARPS * BPW * M), stages it in shared memory with
-// coalesced loads, every warp runs Dykstra for its BPW blocks entirely in
-// registers, hands the log-plan to the rounding stage through shared memory,
-// and the CTA writes whole 32-bit mask words back.
+// Layout in one sentence: a warp owns a unit of BPW consecutive blocks, stages
+// their scores in shared memory with coalesced loads, runs Dykstra for them
+// entirely in registers, hands the log-plan to the rounding stage through shared
+// memory, and writes whole 32-bit mask words back.  Nothing in the method couples
+// two warps, so a CTA is one warp and there is no barrier to wait at (the
+// stopping-test mode at M = 32 excepted, see CtaWarps).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace tsenor {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int WARPS = 4;  // warps per CTA
 
 enum : int { DEV_NONFINITE = 1, DEV_UNDERFILLED = 2, DEV_INTERNAL = 4 };
 
@@ -60,14 +62,15 @@ template <int M_, int V_> struct Geom {
     using T = Tile<M, V>;
     static constexpr int LPB = T::PR * T::PC;        // lanes per block (Dykstra)
     static constexpr int BPW = 32 / LPB;             // blocks per warp
-    static constexpr int PANEL = WARPS * BPW * M;    // panel width in columns
-    static constexpr int WS = PANEL + 1;             // shared row stride (floats)
-    static constexpr int GPW = 32 / M;               // rounding groups per warp
-    static constexpr int PASSES = (BPW + GPW - 1) / GPW;   // rounding passes per warp
-    static constexpr int WORDS = PANEL / 32;         // mask words per panel row
+    static constexpr int UW = BPW * M;               // columns of a unit: its blocks side by side
+    static constexpr int WS = UW + 1;                // shared row stride (floats)
+    static constexpr int GPW = 32 / M;               // rounding groups per warp (blocks of one mask word)
+    static constexpr int PASSES = BPW / GPW;         // rounding passes per warp
+    static constexpr int RO = T::MR / T::PC, CO = T::MC / T::PR;   // lines whose sums a lane finishes
     static_assert(T::MR >= T::PC && T::MC >= T::PR && T::MC % 2 == 0 && (T::MR * T::MC) % 4 == 0, "tile shape");
     static_assert(T::PR * T::MR == M && T::PC * T::MC == M, "tile covers the block");
-    static_assert(WARPS * 32 * T::MR * T::MC <= M * WS, "the per-warp stashes of t0 fit in the key panel");
+    static_assert(BPW % GPW == 0, "a unit is a whole number of mask words wide");
+    static_assert(32 * T::MR * T::MC <= M * WS, "the stash of t0 fits in the key panel");
 };
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -97,8 +100,15 @@ template <int K, int P> __device__ __forceinline__ int xor_perm(int l) {
     return g;
 }
 
-struct OpAdd { __device__ __forceinline__ float operator()(float a, float b) const { return a + b; } };
-struct OpMax { __device__ __forceinline__ float operator()(float a, float b) const { return fmaxf(a, b); } };
+struct OpAdd {
+    static constexpr bool packed = false;
+    __device__ __forceinline__ float operator()(float a, float b) const { return a + b; }
+};
+struct OpAdd2 : OpAdd { static constexpr bool packed = true; };   // pairs by the packed add
+struct OpMax {
+    static constexpr bool packed = false;
+    __device__ __forceinline__ float operator()(float a, float b) const { return fmaxf(a, b); }
+};
 
 // After the call v[0 .. K/P) hold the reduction over the P lanes (lane stride
 // `base`) of the lines those registers stand for.
@@ -108,8 +118,22 @@ __device__ __forceinline__ void reduce_scatter(float (&v)[K], int base, Op op) {
     for (int s = 0; (1 << s) < P; ++s) {
         const int h = K >> (s + 1);
 #pragma unroll
-        for (int k = 0; k < h; ++k)
-            v[k] = op(v[k], __shfl_xor_sync(FULL, v[k + h], base << s));
+        for (int k = 0; k < h; k += 2) {
+            const float x = __shfl_xor_sync(FULL, v[k + h], base << s);
+            if (h == 1) {
+                v[k] = op(v[k], x);
+                continue;
+            }
+            const float y = __shfl_xor_sync(FULL, v[k + 1 + h], base << s);
+            if (Op::packed) {
+                const float2 r = __fadd2_rn(make_float2(v[k], v[k + 1]), make_float2(x, y));
+                v[k] = r.x;
+                v[k + 1] = r.y;
+            } else {
+                v[k] = op(v[k], x);
+                v[k + 1] = op(v[k + 1], y);
+            }
+        }
     }
 }
 // Inverse exchange: v[0 .. K/P) valid on entry, all K valid on return.
@@ -125,16 +149,16 @@ __device__ __forceinline__ void all_gather(float (&v)[K], int base) {
     }
 }
 
-// Kahan-compensated running sum for the few potentials a lane owns.
-struct Comp {
-    float hi, lo;
-    __device__ __forceinline__ void add(float a) {
-        float y = a - lo;
-        float t = hi + y;
-        lo = (t - hi) - y;
-        hi = t;
-    }
-};
+// Adds log2 of a running product of scalings to a Kahan-compensated potential.  The potentials
+// (one row and one column at M = 32) live in shared memory, private to the lane: they are touched
+// once in up to 48 iterations, and without them the loop fits in the 96 registers of 20 warps per SM.
+__device__ __forceinline__ float add_potential(float2* p, float prod) {
+    const float2 c = *p;                     // value, compensation
+    const float y = lg2_approx(prod) - c.y;
+    const float v = c.x + y;
+    *p = make_float2(v, (v - c.x) - y);
+    return v;
+}
 
 // ---------------------------------------------------------------------------
 // Algorithm 1 in potential form, with stabilised linear-domain steps.
@@ -171,7 +195,8 @@ struct Comp {
 // On entry t holds t0 with its row maximum subtracted (exact no-op for the
 // method: the first row projection removes any row constant); on return t
 // holds the final t = x + q.  stash: 32 * MR * MC floats of shared memory
-// private to the warp (keeps t0 while the registers hold U).
+// private to the warp (keeps t0 while the registers hold U); pot: 32 * (RO + CO)
+// float2 of it for the owned potentials.
 // ---------------------------------------------------------------------------
 constexpr int CHECK = 4;     // iterations between range tests of the accumulated scalings
 constexpr int MAXRUN = 48;   // longest run of linear-domain iterations (multiple of CHECK)
@@ -186,55 +211,49 @@ __device__ __forceinline__ bool out_of_window(float p) {
 // issue slots).  The row scalings are never applied to the tile: the registers
 // hold V = U / R_i with R_i the product of the rho_i since the last rebuild, and
 // one multiply per element (by kap_j) is left.  Four fp32 operations per element
-// and iteration, in one of two forms:
-//   SAT  (M >= 16)  rs[a] = R_i:    e = sat(V R_i) = min(U, 1) by a saturating multiply
-//                   (FMA pipe), row sums of e give rho_i = N / sum, column sums are
-//                   sum_i e_ij rho_i, R_i <- R_i rho_i in every lane of the row;
-//   !SAT (M <= 8)   rs[a] = 1/R_i:  m = min(V, 1/R_i) (the clip threshold moves
-//                   instead of the tile), the new R_i is simply N / sum_j m_ij and
-//                   the column sums are sum_i m_ij R_i(new).
-// Both compute the same iterate; which one is faster depends on how the ALU pipe
-// (fp32 min) and the FMA pipe are loaded at that block size (measured).
-template <int M> struct UseSat { static constexpr bool value = (M >= 16); };
+// and iteration: e = sat(V R_i) = min(U, 1) by a saturating multiply, row sums of e
+// give rho_i = N / sum, column sums are sum_i e_ij rho_i, R_i <- R_i rho_i in every
+// lane of the row.  (The other form, min(V, 1/R_i) with the clip threshold moving
+// instead of the tile, needs the half-rate ALU pipe for the min and a second gather
+// for the thresholds: slower at every size, by 3 % for M = 4 and M = 8.)
+//
+// Whether the exchanges' adds and the row factors are packed too is a matter of how the
+// packed and the scalar instructions of the other warps interleave on the FMA pipes, and
+// was measured for each size (1 to 2 %).
+template <int M> struct PackAdd { static constexpr bool value = (M == 8); };
+template <int M> struct PackMul { static constexpr bool value = (M == 8 || M == 32); };
 
 // DELTA: also returns this lane's share of the marginal violation seen by the iteration,
 // max over the lines it owns of |row sum of e - N| and |column sum of e rho - N|.
 template <class G, bool DELTA = false>
 __device__ __forceinline__ float dykstra_step(float2 (&V)[G::T::MR][G::T::MC / 2], float (&rs)[G::T::MR],
-                                              float (&Pr)[G::T::MR / G::T::PC],
-                                              float (&Pc)[G::T::MC / G::T::PR], float Nf, float invN) {
+                                              float (&Pc)[G::CO], float Nf) {
     using T = typename G::T;
     constexpr int M = G::M;
     constexpr int MR = T::MR, MC = T::MC, PR = T::PR, PC = T::PC;
-    constexpr int RO = MR / PC, CO = MC / PR, MP = MC / 2;
-    constexpr bool SAT = UseSat<M>::value;
+    constexpr int RO = G::RO, CO = G::CO, MP = MC / 2;
+    using Add = typename std::conditional<PackAdd<M>::value, OpAdd2, OpAdd>::type;
     float2 m[MR][MP];
-    float rp[MR], sc[MR], thr[MR], cp[MC], kap[MC];
+    float rp[MR], sc[MR], cp[MC], kap[MC];
 #pragma unroll
     for (int a = 0; a < MR; ++a) {
         float2 s2;
 #pragma unroll
         for (int b = 0; b < MP; ++b) {
-            if (SAT) m[a][b] = make_float2(__saturatef(V[a][b].x * rs[a]), __saturatef(V[a][b].y * rs[a]));
-            else m[a][b] = make_float2(fminf(V[a][b].x, rs[a]), fminf(V[a][b].y, rs[a]));
+            m[a][b] = make_float2(__saturatef(V[a][b].x * rs[a]), __saturatef(V[a][b].y * rs[a]));
             s2 = (b == 0) ? m[a][b] : __fadd2_rn(s2, m[a][b]);
         }
         rp[a] = s2.x + s2.y;
     }
-    reduce_scatter<MR, PC>(rp, 1, OpAdd());
+    reduce_scatter<MR, PC>(rp, 1, Add());
     float delta = 0.0f;
-    if (DELTA) {   // row sums of e: rp itself (SAT), rp R_i(old) otherwise
+    if (DELTA) {
 #pragma unroll
-        for (int k = 0; k < RO; ++k) delta = fmaxf(delta, fabsf((SAT ? rp[k] : rp[k] * Pr[k]) - Nf));
+        for (int k = 0; k < RO; ++k) delta = fmaxf(delta, fabsf(rp[k] - Nf));
     }
 #pragma unroll
-    for (int k = 0; k < RO; ++k) {
-        sc[k] = Nf * rcp_approx(rp[k]);          // SAT: rho_i; !SAT: the new R_i
-        if (SAT) Pr[k] *= sc[k];
-        else { Pr[k] = sc[k]; thr[k] = rp[k] * invN; }
-    }
+    for (int k = 0; k < RO; ++k) sc[k] = Nf * rcp_approx(rp[k]);
     all_gather<MR, PC>(sc, 1);
-    if (!SAT) all_gather<MR, PC>(thr, 1);
 #pragma unroll
     for (int b = 0; b < MP; ++b) {
         float2 c2 = __fmul2_rn(m[0][b], make_float2(sc[0], sc[0]));
@@ -243,7 +262,7 @@ __device__ __forceinline__ float dykstra_step(float2 (&V)[G::T::MR][G::T::MC / 2
         cp[2 * b] = c2.x;
         cp[2 * b + 1] = c2.y;
     }
-    reduce_scatter<MC, PR>(cp, PC, OpAdd());
+    reduce_scatter<MC, PR>(cp, PC, Add());
     if (DELTA) {
 #pragma unroll
         for (int k = 0; k < CO; ++k) delta = fmaxf(delta, fabsf(cp[k] - Nf));
@@ -254,30 +273,40 @@ __device__ __forceinline__ float dykstra_step(float2 (&V)[G::T::MR][G::T::MC / 2
         Pc[k] *= kap[k];
     }
     all_gather<MC, PR>(kap, PC);
+    if constexpr (PackMul<M>::value && MR % 2 == 0) {
 #pragma unroll
-    for (int a = 0; a < MR; ++a) {
-        if (SAT) rs[a] *= sc[a];
-        else rs[a] = thr[a];
+        for (int a = 0; a < MR; a += 2) {
+            const float2 r = __fmul2_rn(make_float2(rs[a], rs[a + 1]), make_float2(sc[a], sc[a + 1]));
+            rs[a] = r.x;
+            rs[a + 1] = r.y;
+        }
+    } else {
+#pragma unroll
+        for (int a = 0; a < MR; ++a) rs[a] *= sc[a];
+    }
+#pragma unroll
+    for (int a = 0; a < MR; ++a)
 #pragma unroll
         for (int b = 0; b < MP; ++b) V[a][b] = __fmul2_rn(V[a][b], make_float2(kap[2 * b], kap[2 * b + 1]));
-    }
     return delta;
 }
 
-// Returns the number of iterations run: iters, or fewer in the stopping-test mode (ee_eps > 0):
+// Returns the number of iterations run: iters, or fewer in the stopping-test mode (EE, ee_eps > 0):
 // after every group of CHECK iterations, i.e. at iterations 5, 9, 13, ... of Algorithm 1, the
 // warp stops once the marginal violation of every block it holds is below ee_eps.
-template <class G>
-__device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], float* stash, int lane,
+template <class G, bool EE>
+__device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], float* stash, float2* pot, int lane,
                                                float Nf, float log2N, int iters, float ee_eps) {
     using T = typename G::T;
     constexpr int MR = T::MR, MC = T::MC, PR = T::PR, PC = T::PC;
-    constexpr int RO = MR / PC, CO = MC / PR;  // lines whose sums this lane finishes
+    constexpr int RO = G::RO, CO = G::CO;
     constexpr int MP = MC / 2, NQ = MR * MC / 4;
     float F[MR], Gc[MC];
-    Comp Fo[RO], Go[CO];
-    float Pr[RO], Pc[CO];                      // products of rho / kap since the last rebuild
+    float rs[MR];
+    float Pc[CO];              // products of kap since the last rebuild; those of rho are rs[0 .. RO)
     if (iters <= 0) return 0;
+    float2* const fpot = pot + lane;                 // the owned potentials, compensated
+    float2* const gpot = pot + RO * 32 + lane;
     float4* const st4 = reinterpret_cast<float4*>(stash) + lane;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {   // sub-tile in row-major order, four elements per slot
@@ -297,10 +326,9 @@ __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], f
         reduce_scatter<MR, PC>(rp, 1, OpAdd());
 #pragma unroll
         for (int k = 0; k < RO; ++k) {
-            Fo[k].hi = log2N - lg2_approx(rp[k]);
-            Fo[k].lo = 0.f;
-            F[k] = Fo[k].hi;
-            Pr[k] = 1.0f;
+            F[k] = log2N - lg2_approx(rp[k]);
+            fpot[k * 32] = make_float2(F[k], 0.f);
+            rs[k] = 1.0f;
         }
         all_gather<MR, PC>(F, 1);
         float cm[MC];
@@ -324,23 +352,20 @@ __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], f
         reduce_scatter<MC, PR>(cp, PC, OpAdd());
 #pragma unroll
         for (int k = 0; k < CO; ++k) {
-            Go[k].hi = (log2N - cm[k]) - lg2_approx(cp[k]);
-            Go[k].lo = 0.f;
+            gpot[k * 32] = make_float2((log2N - cm[k]) - lg2_approx(cp[k]), 0.f);
             Pc[k] = 1.0f;
         }
     }
     // Iterations 1 .. iters-1 in runs: rebuild U from the potentials, then groups of
     // CHECK iterations with the range test of the accumulated scalings between groups.
     float2 V[MR][MP];
-    float rs[MR];
-    const float invN = 1.0f / Nf;
     int it = 1;
 #pragma unroll 1
     while (it < iters) {
 #pragma unroll
-        for (int k = 0; k < RO; ++k) { Fo[k].add(lg2_approx(Pr[k])); Pr[k] = 1.0f; F[k] = Fo[k].hi; }
+        for (int k = 0; k < RO; ++k) F[k] = add_potential(fpot + k * 32, rs[k]);
 #pragma unroll
-        for (int k = 0; k < CO; ++k) { Go[k].add(lg2_approx(Pc[k])); Pc[k] = 1.0f; Gc[k] = Go[k].hi; }
+        for (int k = 0; k < CO; ++k) { Gc[k] = add_potential(gpot + k * 32, Pc[k]); Pc[k] = 1.0f; }
         all_gather<MR, PC>(F, 1);
         all_gather<MC, PR>(Gc, PC);
 #pragma unroll
@@ -355,15 +380,15 @@ __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], f
             V[a1][b1 / 2] = make_float2(ex2_approx(x1.x), ex2_approx(x1.y));
         }
 #pragma unroll
-        for (int a = 0; a < MR; ++a) rs[a] = 1.0f;     // R_i = 1 (and 1/R_i = 1)
+        for (int a = 0; a < MR; ++a) rs[a] = 1.0f;     // R_i = 1
         const int run_end = (iters - it > MAXRUN) ? it + MAXRUN : iters;
         bool wide = false;
 #pragma unroll 1
         while (!wide && it + CHECK <= run_end) {
-#pragma unroll(G::M == 8 ? 1 : CHECK)   // measured: unrolling the group helps every size but M = 8
-            for (int u = 0; u < CHECK - 1; ++u) dykstra_step<G>(V, rs, Pr, Pc, Nf, invN);
-            if (ee_eps > 0.0f) {
-                const float delta = dykstra_step<G, true>(V, rs, Pr, Pc, Nf, invN);
+#pragma unroll(EE && G::M == 32 ? 1 : CHECK)   // (the stopping test at M = 32 is mostly code that runs once)
+            for (int u = 0; u < CHECK - 1; ++u) dykstra_step<G>(V, rs, Pc, Nf);
+            if constexpr (EE) {
+                const float delta = dykstra_step<G, true>(V, rs, Pc, Nf);
                 if (__all_sync(FULL, delta < ee_eps)) {   // every block of the warp has converged
                     it += CHECK;
                     iters = it;
@@ -371,7 +396,7 @@ __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], f
                     break;
                 }
             } else {
-                dykstra_step<G>(V, rs, Pr, Pc, Nf, invN);
+                dykstra_step<G>(V, rs, Pc, Nf);
             }
             it += CHECK;
             // exponent field in [127-16, 127+16] <=> product in [2^-16, 2^17).  A product that
@@ -379,21 +404,21 @@ __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], f
             // not vote, so that it cannot change when the other blocks of its warp rebuild.
             bool w = false;
 #pragma unroll
-            for (int k = 0; k < RO; ++k) w |= out_of_window(Pr[k]);
+            for (int k = 0; k < RO; ++k) w |= out_of_window(rs[k]);
 #pragma unroll
             for (int k = 0; k < CO; ++k) w |= out_of_window(Pc[k]);
             wide = __any_sync(FULL, w);
         }
         if (!wide) {   // fewer than CHECK iterations left (end of the last run only)
 #pragma unroll 1
-            for (; it < run_end; ++it) dykstra_step<G>(V, rs, Pr, Pc, Nf, invN);
+            for (; it < run_end; ++it) dykstra_step<G>(V, rs, Pc, Nf);
         }
     }
     // final potentials and t = t0 + F + G
 #pragma unroll
-    for (int k = 0; k < RO; ++k) { Fo[k].add(lg2_approx(Pr[k])); F[k] = Fo[k].hi; }
+    for (int k = 0; k < RO; ++k) F[k] = add_potential(fpot + k * 32, rs[k]);
 #pragma unroll
-    for (int k = 0; k < CO; ++k) { Go[k].add(lg2_approx(Pc[k])); Gc[k] = Go[k].hi; }
+    for (int k = 0; k < CO; ++k) Gc[k] = add_potential(gpot + k * 32, Pc[k]);
     all_gather<MR, PC>(F, 1);
     all_gather<MC, PR>(Gc, PC);
 #pragma unroll
@@ -471,77 +496,126 @@ __device__ __forceinline__ float4 load_score_quad(const ScoreSrc& S, int64_t r, 
 __device__ __forceinline__ int any_nan(const float4& v) {
     return !(v.x == v.x) | !(v.y == v.y) | !(v.z == v.z) | !(v.w == v.w);
 }
-__device__ __forceinline__ int any_nonfinite(const float4& v) {
-    return !(fabsf(v.x) <= 3.4028234e38f) | !(fabsf(v.y) <= 3.4028234e38f) |
-           !(fabsf(v.z) <= 3.4028234e38f) | !(fabsf(v.w) <= 3.4028234e38f);
+// ---------------------------------------------------------------------------
+// Where a unit's blocks live in the matrix.  The blocks of the matrix are numbered
+// row by row, every block row padded to a whole number of mask words (`nbp` slots of
+// which `nbc` hold blocks; a single block column, as in the column groups of
+// SparseGPT, is not padded), and a unit is BPW consecutive slots: it runs on into the
+// next block row where one ends, so ragged widths and slabs fill their warps too.  In
+// shared memory slot b of the unit occupies columns [b M, b M + M).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ int64_t div_slots(int64_t a, int64_t b) {   // 0 <= a, 0 < b
+    return (((uint64_t)a | (uint64_t)b) >> 32) ? a / b : (int64_t)((unsigned)a / (unsigned)b);
 }
-
-// ---------------------------------------------------------------------------
-// Where a panel's cells live in the matrix.  Wide matrices: the panel is M rows
-// x PANEL columns at (r0, c0).  Slabs (a single block column, cols == M, as in
-// the column groups of SparseGPT): the panel's blocks are stacked vertically,
-// block b of the panel being rows [(first + b) M, (first + b + 1) M), so that a
-// CTA still gets a full set of blocks and the whole slab is one wave of CTAs.
-// In shared memory both look the same: block b occupies columns [b M, b M + M).
-// ---------------------------------------------------------------------------
-template <int M> struct PanelMap {
-    int tall;
-    int64_t r0, c0;        // wide: origin of the panel
-    int64_t first;         // tall: first block (= block row) of the panel
-    int valid_cols;        // columns of the shared-memory panel that hold blocks
+// Volatile: read again where it is needed, so that no position in the matrix stays in registers
+// over the iterations.
+__device__ __forceinline__ int64_t this_cta() {
+    unsigned u;
+    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(u));
+    return u;
+}
+template <int WPC> __device__ __forceinline__ int64_t this_unit() {
+    return this_cta() * WPC + threadIdx.x / 32;
+}
+template <int M> struct UnitMap {
     int64_t rows, cols;    // extent of the matrix
+    int64_t nbc, nbp;      // blocks per block row, and slots
+    int64_t bi0, bj0;      // block row and slot of the unit's first slot
+    __device__ __forceinline__ UnitMap(int64_t rows_, int64_t cols_, int64_t nbp_, int64_t first)
+        : rows(rows_), cols(cols_), nbc(cols_ / M), nbp(nbp_) {
+        bi0 = div_slots(first, nbp_);
+        bj0 = first - bi0 * nbp_;
+    }
+    // Origin of slot b of the unit; false if there is no such block.
+    __device__ __forceinline__ bool locate(int b, int64_t& r0, int64_t& c0) const {
+        int64_t bi = bi0, bj = bj0 + b;
+        if (bj >= nbp) {                     // the unit ran on into a later block row
+            const int64_t q = div_slots(bj, nbp);
+            bi += q;
+            bj -= q * nbp;
+        }
+        r0 = bi * M;
+        c0 = bj * M;
+        return r0 < rows && bj < nbc;
+    }
     __device__ __forceinline__ bool holds_quad(int64_t r, int64_t c) const {
         return r >= 0 && r < rows && c >= 0 && c + 4 <= cols;
     }
-    __device__ __forceinline__ int64_t row(int r, int c) const { return tall ? (first + c / M) * M + r : r0 + r; }
-    __device__ __forceinline__ int64_t col(int c) const { return tall ? (int64_t)(c % M) : c0 + c; }
 };
 
 // ---------------------------------------------------------------------------
-// Panel loaders: an M x PANEL panel into shared memory, coalesced, vector
-// loads when the addresses allow it.  Return non-zero if this thread saw a
+// Unit loaders: COLS columns (from slot `slot0` on) of the unit's M rows into shared memory
+// (dst: row stride WS), coalesced, vector loads when the addresses allow it.  A lane keeps its
+// column(s) and walks down the rows, BATCH of them in flight: the position is worked out once.
+// The common source (fp32 |W|, aligned) has a loop of its own with every load in flight; the
+// others share one that is unrolled less, because the instruction cache is what the warps of
+// an SM, spread over all phases of the kernel, compete for.  Return non-zero if this lane saw a
 // non-finite score, respectively a NaN key.
 // ---------------------------------------------------------------------------
-template <class G>
-__device__ __forceinline__ int load_score_panel(const ScoreSrc& S, const PanelMap<G::M>& pm,
-                                                float* __restrict__ dst) {
+template <class G, int COLS, int BATCH, class Load>
+__device__ __forceinline__ void load_unit(const UnitMap<G::M>& um, int slot0, int lane, float* __restrict__ dst,
+                                          Load load) {
     constexpr int M = G::M;
-    constexpr int V = G::PANEL / 4;
-    int bad = 0;
-    for (int idx = threadIdx.x; idx < M * V; idx += WARPS * 32) {
-        const int r = idx / V, c = (idx % V) * 4;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c < pm.valid_cols && TS_CHECK(pm.holds_quad(pm.row(r, c), pm.col(c))))
-            v = load_score_quad(S, pm.row(r, c), pm.col(c));  // a quad is all in or all out
-        bad |= any_nonfinite(v);
-        if (TS_CHECK(r < M && c + 4 <= G::PANEL)) {
-            float* d = dst + r * G::WS + c;
-            d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
+    constexpr int QW = (COLS / 4 < 32) ? COLS / 4 : 32;     // quads of a row that the warp takes at once
+    constexpr int RPI = 32 / QW, STEPS = M / RPI;           // rows it takes at once
+    constexpr int B = (BATCH < STEPS) ? BATCH : STEPS;
+    static_assert(M % RPI == 0 && STEPS % B == 0, "whole batches");
+#pragma unroll 1
+    for (int cs = 0; cs < COLS / (4 * QW); ++cs) {
+        const int c = (lane % QW + cs * QW) * 4;
+        int64_t r0, c0;
+        const bool there = um.locate(slot0 + c / M, r0, c0);
+        r0 += lane / QW;
+        c0 += c % M;
+        float* d = dst + (lane / QW) * G::WS + c;
+#pragma unroll 1
+        for (int i0 = 0; i0 < STEPS; i0 += B, r0 += B * RPI, d += B * RPI * G::WS) {
+            float4 v[B];
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (there && TS_CHECK(um.holds_quad(r0 + i * RPI, c0))) v[i] = load(r0 + i * RPI, c0);
+            }
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                if (!TS_CHECK(lane / QW + (i0 + i) * RPI < M && c + 4 <= G::UW)) continue;
+                float* const e = d + i * RPI * G::WS;
+                e[0] = v[i].x; e[1] = v[i].y; e[2] = v[i].z; e[3] = v[i].w;
+            }
         }
     }
-    return bad;
 }
-
-template <class G>
-__device__ __forceinline__ int load_key_panel(const float* __restrict__ src, int64_t ld, const PanelMap<G::M>& pm,
-                                              bool vec_ok, float* __restrict__ dst) {
-    constexpr int M = G::M;
-    constexpr int V = G::PANEL / 4;
-    int bad = 0;
-    for (int idx = threadIdx.x; idx < M * V; idx += WARPS * 32) {
-        const int r = idx / V, c = (idx % V) * 4;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c < pm.valid_cols && TS_CHECK(pm.holds_quad(pm.row(r, c), pm.col(c)))) {
-            const float* p = src + pm.row(r, c) * ld + pm.col(c);
-            if (vec_ok) v = __ldg(reinterpret_cast<const float4*>(p));
-            else v = make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
-        }
-        bad |= any_nan(v);          // infinite keys have a place in the order; NaN keys are flagged
-        if (TS_CHECK(r < M && c + 4 <= G::PANEL)) {
-            float* d = dst + r * G::WS + c;
-            d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
-        }
+template <class G, int COLS>
+__device__ __forceinline__ int load_scores(const ScoreSrc& S, const UnitMap<G::M>& um, int slot0, int lane,
+                                           float* __restrict__ dst) {
+    float nan = 0.0f;     // 0 x is a NaN for a non-finite x
+    const auto seen = [&](const float4& v) {
+        nan = fmaf(v.x, 0.0f, fmaf(v.y, 0.0f, fmaf(v.z, 0.0f, fmaf(v.w, 0.0f, nan))));
+        return v;
+    };
+    if (S.kind == SC_ABS && !S.w_is_bf16 && S.vec_w) {
+        const float* const w = static_cast<const float*>(S.w);
+        load_unit<G, COLS, 8>(um, slot0, lane, dst, [&](int64_t r, int64_t c) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(w + r * S.ld + c));
+            return seen(make_float4(fabsf(v.x), fabsf(v.y), fabsf(v.z), fabsf(v.w)));
+        });
+    } else {
+        load_unit<G, COLS, 2>(um, slot0, lane, dst,
+                              [&](int64_t r, int64_t c) { return seen(load_score_quad(S, r, c)); });
     }
+    return nan != 0.0f;
+}
+template <class G>
+__device__ __forceinline__ int load_keys(const float* __restrict__ src, int64_t ld, const UnitMap<G::M>& um,
+                                         bool vec_ok, int lane, float* __restrict__ dst) {
+    int bad = 0;
+    load_unit<G, G::UW, 4>(um, 0, lane, dst, [&](int64_t r, int64_t c) {
+        const float* p = src + r * ld + c;
+        const float4 v = vec_ok ? __ldg(reinterpret_cast<const float4*>(p))
+                                : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+        bad |= any_nan(v);          // infinite keys have a place in the order; NaN keys are flagged
+        return v;
+    });
     return bad;
 }
 
@@ -559,22 +633,22 @@ __device__ __forceinline__ int load_key_panel(const float* __restrict__ src, int
 //   M <= 16:  [0,2M) row prefixes of row i, [2M,4M) column prefixes of column i
 constexpr int CPRE_STRIDE = 33;   // words per column-prefix table at M = 32 (odd: conflict-free)
 
-// Strict order "key descending, index ascending" as one ascending u64.
-__device__ __forceinline__ unsigned long long sort_word(float key, int idx) {
-    if (!(key == key)) key = __int_as_float(0xff800000);  // NaN orders as -inf
-    key += 0.0f;                                          // -0 -> +0
-    unsigned u = __float_as_uint(key);
-    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);       // ascending uint == ascending float
-    return ((unsigned long long)(~u) << 32) | (unsigned)idx;
+// The strict order "key descending, index ascending": ascending words of the key; NaN orders as
+// -inf, -0 as +0.
+__device__ __forceinline__ unsigned order_word(float key) {
+    if (!(key == key)) key = __int_as_float(0xff800000);
+    key += 0.0f;
+    const unsigned u = __float_as_uint(key);
+    return (u & 0x80000000u) ? u : ~(u | 0x80000000u);
 }
 
-// The same order packed into one ascending 32-bit word: the high word of sort_word with its
-// five low bits replaced by the index.  Dropping those bits is harmless unless two keys of
-// the line agree in the 27 bits kept ("same bucket"): then their order may depend on the
-// bits dropped, and the caller falls back to the 64-bit words.  Keys that are exactly zero
-// (the capped entries of a plan: up to half of a line) are the one common case of equal
-// keys; each of them gets a bucket of its own, ZERO_BUCKET + index (zeros order among
-// themselves by index), and the positive keys are shifted down by the 32 buckets this takes.
+// That order packed into one ascending 32-bit word: order_word with its five low bits replaced by
+// the index.  Dropping those bits is harmless unless two keys of the line agree in the 27 bits kept
+// ("same bucket"): the network then leaves them side by side in index order, and sort_line puts
+// them right by their full keys.  Keys that are exactly zero (the capped entries of a plan: up to
+// half of a line) are the one common case of equal keys; each of them gets a bucket of its own,
+// ZERO_BUCKET + index (zeros order among themselves by index), and the positive keys are shifted
+// down by the 32 buckets this takes.
 constexpr unsigned ZERO_BUCKET = 0x03ffffe0u;
 __device__ __forceinline__ unsigned sort_word_packed(float key, unsigned idx) {
     if (!(key == key)) key = __int_as_float(0xff800000);
@@ -586,82 +660,91 @@ __device__ __forceinline__ unsigned sort_word_packed(float key, unsigned idx) {
     else hi = 0x7fffffffu - b - (32u * 32u + 31u);             // positive: larger first, all before the zeros
     return (hi & ~31u) | idx;
 }
+// The same word for a key that is known to be <= 0 and not NaN (every entry of a capped log-plan).
+__device__ __forceinline__ unsigned sort_word_capped(float key, unsigned idx) {
+    const unsigned hi = (key == 0.0f) ? (ZERO_BUCKET + idx) << 5 : __float_as_uint(key);
+    return (hi & ~31u) | idx;
+}
 
 // Batcher's odd-even merge sort as a fully unrolled network (191 compare-exchanges for 32
 // keys, 63 for 16, 19 for 8, 5 for 4), ascending.  Indices are template constants so that the
-// keys stay in registers.  A compare-exchange costs two instructions on 32-bit words (min,
-// max) and six on 64-bit words.
-template <int I, int J, int M> __device__ __forceinline__ void cmp_swap(unsigned long long (&v)[M]) {
-    const unsigned long long a = v[I], b = v[J];
-    const bool sw = a > b;
-    v[I] = sw ? b : a;
-    v[J] = sw ? a : b;
-}
+// keys stay in registers.  A compare-exchange is a min and a max.
 template <int I, int J, int M> __device__ __forceinline__ void cmp_swap(unsigned (&v)[M]) {
     const unsigned a = v[I], b = v[J];
     v[I] = min(a, b);
     v[J] = max(a, b);
 }
-template <int LO, int N, int R, int I, class T, int M> __device__ __forceinline__ void oem_chain(T (&v)[M]) {
+template <int LO, int N, int R, int I, int M> __device__ __forceinline__ void oem_chain(unsigned (&v)[M]) {
     if constexpr (I + R < LO + N) {
         cmp_swap<I, I + R, M>(v);
-        oem_chain<LO, N, R, I + 2 * R, T, M>(v);
+        oem_chain<LO, N, R, I + 2 * R, M>(v);
     }
 }
 // merges the two sorted halves of the subsequence LO, LO+R, LO+2R, ... of v[LO .. LO+N)
-template <int LO, int N, int R, class T, int M> __device__ __forceinline__ void oem_merge(T (&v)[M]) {
+template <int LO, int N, int R, int M> __device__ __forceinline__ void oem_merge(unsigned (&v)[M]) {
     if constexpr (2 * R < N) {
-        oem_merge<LO, N, 2 * R, T, M>(v);
-        oem_merge<LO + R, N, 2 * R, T, M>(v);
-        oem_chain<LO, N, R, LO + R, T, M>(v);
+        oem_merge<LO, N, 2 * R, M>(v);
+        oem_merge<LO + R, N, 2 * R, M>(v);
+        oem_chain<LO, N, R, LO + R, M>(v);
     } else {
         cmp_swap<LO, LO + R, M>(v);
     }
 }
-template <int LO, int N, class T, int M> __device__ __forceinline__ void oem_sort(T (&v)[M]) {
+template <int LO, int N, int M> __device__ __forceinline__ void oem_sort(unsigned (&v)[M]) {
     if constexpr (N > 1) {
-        oem_sort<LO, N / 2, T, M>(v);
-        oem_sort<LO + N / 2, N / 2, T, M>(v);
-        oem_merge<LO, N, 1, T, M>(v);
+        oem_sort<LO, N / 2, M>(v);
+        oem_sort<LO + N / 2, N / 2, M>(v);
+        oem_merge<LO, N, 1, M>(v);
     }
 }
-template <class T, int M> __device__ __forceinline__ void sort_regs(T (&v)[M]) { oem_sort<0, M, T, M>(v); }
 
-// Sorts one line (stride `st` floats in shared memory) and returns the prefix sets of the
-// sorted order: pre[p] = positions of the p+1 best entries, packed two per word (16 bits
-// each) for M <= 16.
-template <int M> struct PreWords { static constexpr int value = (M == 32) ? 32 : M / 2; };
-template <int M, class T>
-__device__ __forceinline__ void prefix_sets(const T (&v)[M], unsigned (&pre)[PreWords<M>::value]) {
+// Sorts one line, given its keys in registers and its place in shared memory (stride `st`
+// floats): on return the low five bits of w[p] are the position of the p-th best entry.
+// capped: the keys are known to be <= 0 and not NaN.
+template <int M>
+__device__ __forceinline__ void sort_line(const float (&key)[M], const float* line, int st, bool capped,
+                                          unsigned (&w)[M]) {
+    if (capped) {
+#pragma unroll
+        for (int k = 0; k < M; ++k) w[k] = sort_word_capped(key[k], k);
+    } else {
+#pragma unroll
+        for (int k = 0; k < M; ++k) w[k] = sort_word_packed(key[k], k);
+    }
+    oem_sort<0, M, M>(w);
+    unsigned closest = 0xffffffffu;     // smallest difference pattern of two neighbours
+#pragma unroll
+    for (int p = 0; p + 1 < M; ++p) closest = min(closest, w[p] ^ w[p + 1]);
+    // Rare: two non-zero keys of a line within 2^-18 of each other.  Passes of neighbour exchanges
+    // among the entries of a bucket, by full key, until nothing moves: a bucket of L entries is
+    // in order after at most L - 1 of them (entries of different buckets, and equal keys, stay as
+    // they are).  A sixth of the code of a second network on 64-bit words, and a fifth of its time.
+    bool more = closest < 32u;
+#pragma unroll 1
+    for (int pass = 0; pass < M && __any_sync(FULL, more); ++pass) {
+        bool moved = false;
+#pragma unroll
+        for (int p = 0; p + 1 < M; ++p) {
+            if (more && (w[p] ^ w[p + 1]) < 32u) {
+                const unsigned a = w[p], b = w[p + 1];
+                if (order_word(line[(b & 31u) * st]) < order_word(line[(a & 31u) * st])) {
+                    w[p] = b;
+                    w[p + 1] = a;
+                    moved = true;
+                }
+            }
+        }
+        more = moved;
+    }
+}
+// Prefix sets of a sorted line, for M <= 16 two to a word: pre[p] = positions of the p+1 best.
+template <int M> __device__ __forceinline__ void prefix_sets(const unsigned (&w)[M], unsigned (&pre)[M / 2]) {
     unsigned acc = 0u;
 #pragma unroll
     for (int p = 0; p < M; ++p) {
-        acc |= 1u << ((unsigned)v[p] & 31u);
-        if (M == 32) pre[p] = acc;
-        else if (p % 2 == 0) pre[p / 2] = acc;
+        acc |= 1u << (w[p] & 31u);
+        if (p % 2 == 0) pre[p / 2] = acc;
         else pre[p / 2] |= acc << 16;
-    }
-}
-template <int M>
-__device__ __forceinline__ void sort_line(const float* line, int st, unsigned (&pre)[PreWords<M>::value]) {
-    bool same_bucket;
-    {   // fast path: packed 32-bit words
-        unsigned w[M];
-#pragma unroll
-        for (int k = 0; k < M; ++k) w[k] = sort_word_packed(line[k * st], k);
-        sort_regs(w);
-        unsigned closest = 0xffffffffu;     // smallest difference pattern of two neighbours
-#pragma unroll
-        for (int p = 0; p + 1 < M; ++p) closest = min(closest, w[p] ^ w[p + 1]);
-        same_bucket = closest < 32u;
-        prefix_sets<M>(w, pre);
-    }
-    if (__any_sync(FULL, same_bucket)) {   // rare: two non-zero keys of a line within 2^-18 of each other
-        unsigned long long v[M];
-#pragma unroll
-        for (int k = 0; k < M; ++k) v[k] = sort_word(line[k * st], k);
-        sort_regs(v);
-        prefix_sets<M>(v, pre);
     }
 }
 
@@ -706,11 +789,13 @@ template <int M> __device__ __forceinline__ unsigned transpose_bits(unsigned x, 
 //   ks, ws: shared-memory pointers to element (0,0) of the block's keys and
 //   |scores| (row stride WS); the key cells are overwritten.  cpre: this
 //   lane's column-prefix table when it does not fit in the key cells (M = 32).
-//   active: group has a block.
+//   active: group has a block.  capped: the keys are known to be <= 0.  before_search: called
+//   by the whole warp, once the tables are done with, if ws is going to be read.
 // Returns this lane's row of the mask (M bits).  flags accumulates DEV_* bits.
-template <class G>
+template <class G, class BeforeSearch>
 __device__ __forceinline__ unsigned round_block(float* ks, const float* ws, unsigned* cpre, int lane, bool active,
-                                                int N, int ls_steps, int& flags) {
+                                                bool capped, int N, int ls_steps, int& flags,
+                                                BeforeSearch before_search) {
     constexpr int M = G::M;
     constexpr int WS = G::WS;
     constexpr unsigned GM = (M == 32) ? 0xffffffffu : ((1u << (M & 31)) - 1u);
@@ -720,22 +805,49 @@ __device__ __forceinline__ unsigned round_block(float* ks, const float* ws, unsi
     // ---- sorted orders of my row and of my column (Algorithm 2 line 2), kept as prefix sets
     unsigned char* const rtab = reinterpret_cast<unsigned char*>(ks + i * WS);
     unsigned char* const ctab = (M == 32) ? reinterpret_cast<unsigned char*>(cpre) : rtab + 2 * M;
-    {
-        constexpr int PW = PreWords<M>::value;
-        unsigned pc[PW];
-        sort_line<M>(ks + i, WS, pc);
-        if (M == 32) {                      // not aliased with the keys: store at once
+    if constexpr (M == 32) {
+        // One sort body for both sides: the network is some 900 instructions long and the warps of an
+        // SM are spread over the whole kernel, so what counts is that its code stays in the cache.
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+            float key[M];
+            unsigned w[M];
+            if (side == 0) {
 #pragma unroll
-            for (int w = 0; w < PW; ++w) reinterpret_cast<unsigned*>(ctab)[w] = pc[w];
+                for (int k = 0; k < M; ++k) key[k] = ks[k * WS + i];
+            } else {
+#pragma unroll
+                for (int k = 0; k < M; ++k) key[k] = ks[i * WS + k];
+            }
+            sort_line<M>(key, side ? ks + i * WS : ks + i, side ? 1 : WS, capped, w);
+            __syncwarp();                   // side 1: every lane is done reading keys
+            unsigned* const tab = reinterpret_cast<unsigned*>(side ? rtab : ctab);
+            unsigned acc = 0u;
+#pragma unroll
+            for (int p = 0; p < M; ++p) {
+                acc |= 1u << (w[p] & 31u);
+                tab[p] = acc;
+            }
         }
-        unsigned pr[PW];
-        sort_line<M>(ks + i * WS, 1, pr);
+    } else {
+        unsigned pc[M / 2], pr[M / 2];
+        {
+            float key[M];
+            unsigned w[M];
+#pragma unroll
+            for (int k = 0; k < M; ++k) key[k] = ks[k * WS + i];
+            sort_line<M>(key, ks + i, WS, capped, w);
+            prefix_sets<M>(w, pc);
+#pragma unroll
+            for (int k = 0; k < M; ++k) key[k] = ks[i * WS + k];
+            sort_line<M>(key, ks + i * WS, 1, capped, w);
+            prefix_sets<M>(w, pr);
+        }
         __syncwarp();                       // every lane is done reading keys
 #pragma unroll
-        for (int w = 0; w < PW; ++w) reinterpret_cast<unsigned*>(rtab)[w] = pr[w];
-        if (M != 32) {
-#pragma unroll
-            for (int w = 0; w < PW; ++w) reinterpret_cast<unsigned*>(ctab)[w] = pc[w];
+        for (int w = 0; w < M / 2; ++w) {
+            reinterpret_cast<unsigned*>(rtab)[w] = pr[w];
+            reinterpret_cast<unsigned*>(ctab)[w] = pc[w];
         }
     }
     __syncwarp();
@@ -756,9 +868,18 @@ __device__ __forceinline__ unsigned round_block(float* ks, const float* ws, unsi
         if (round == M * M - 1) flags |= DEV_INTERNAL;
         const unsigned pickR = first_available<M>(availR, capR, rtab);
         const unsigned pickC = first_available<M>(availC, capC, ctab);
-        // an entry picked from both sides is taken
-        const unsigned takenR = pickR & transpose_bits<M>(pickC, i);   // columns taken in my row
-        const unsigned takenC = transpose_bits<M>(takenR, i);          // rows taken in my column
+        // an entry picked from both sides is taken: takenR columns in my row, takenC rows in my
+        // column.  (Both picks are transposed, not takenR a second time: two chains of five
+        // exchanges side by side, or one for M <= 16, where both fit into one word.)
+        unsigned takenR, takenC;
+        if (M == 32) {
+            takenR = pickR & transpose_bits<M>(pickC, i);
+            takenC = pickC & transpose_bits<M>(pickR, i);
+        } else {
+            const unsigned tt = transpose_bits<M>(pickC | (pickR << 16), i);
+            takenR = pickR & tt;
+            takenC = pickC & (tt >> 16);
+        }
         sel |= takenR;
         selC |= takenC;
         capR -= __popc(takenR);
@@ -773,6 +894,7 @@ __device__ __forceinline__ unsigned round_block(float* ks, const float* ws, unsi
     // ---- local search (lines 7-13, Eq. 6).  sel: my row of the mask (bits over columns);
     // selC: my column (bits over rows).  Lane j' scans the rows i' that can form a valid
     // triple with it: S[i'][j'] = 1 and S[i'][j] = 0, provided S[i][j'] = 0.
+    if (ls_steps != 0 && __any_sync(FULL, capR > 0)) before_search();
     bool stopped = !active;
     int steps = 0;
     for (int it = 0; it <= M * N; ++it) {
@@ -835,8 +957,7 @@ struct Params {
     float* plan;         int64_t ld_plan; int plan_is_log;
     uint32_t* bits;      int64_t wpr;
     int64_t rows, cols;
-    int npc;                       // panels per block row
-    int tall;                      // slab: one block column, panels stacked vertically
+    int64_t nbp;                   // slots of a block row (see UnitMap)
     int N; float Nf, log2N;
     float c_hi, c_lo;              // tau * log2(e), split in two floats
     int per_block_tau;             // tau is divided by each block's own largest score
@@ -844,82 +965,112 @@ struct Params {
     float ee_eps;                  // > 0: stopping test of Algorithm 1 (non-parity mode)
     unsigned long long* iter_sum;  // optional: iterations run, summed over the blocks
     int32_t* status;
-    int vec_keys;
+    int vec_keys, vec_plan;
 };
 
-template <class G, int MODE> struct SmemLayout {
-    static constexpr int M = G::M;
-    float w[M * G::WS];
-    float k[M * G::WS];
-    unsigned int bits[M * G::WORDS];
-    unsigned int cpre[(M == 32) ? WARPS * 32 * CPRE_STRIDE : 1];   // column-prefix tables (M = 32)
-};
-template <class G> struct SmemLayout<G, 1> {   // Algorithm 1 alone: score panel and the t0 stash
-    static constexpr int M = G::M;
-    float w[M * G::WS];
-    float k[WARPS * 32 * G::T::MR * G::T::MC];
-    unsigned int bits[1];
-    unsigned int cpre[1];
-};
-// Resident CTAs per SM the register allocation aims for.
-template <int M, int V> struct MinBlocks { static constexpr int value = (V == 1) ? 4 : (M == 4) ? 5 : 4; };
+// The plan of a unit from shared memory to the matrix, whole rows of the unit at a time.
+template <class G>
+__device__ __forceinline__ void store_plan(const Params& P, const UnitMap<G::M>& um, int lane, const float* src) {
+    constexpr int M = G::M;
+    constexpr int QW = (G::UW / 4 < 32) ? G::UW / 4 : 32, RPI = 32 / QW;
+#pragma unroll 1
+    for (int cs = 0; cs < G::UW / (4 * QW); ++cs) {
+        const int c = (lane % QW + cs * QW) * 4;
+        int64_t r0, c0;
+        if (!um.locate(c / M, r0, c0)) continue;
+#pragma unroll 2
+        for (int r = lane / QW; r < M; r += RPI) {
+            if (!TS_CHECK(c + 4 <= G::UW && um.holds_quad(r0 + r, c0 + c % M))) continue;
+            const float* const k = src + r * G::WS + c;
+            float4 v = make_float4(k[0], k[1], k[2], k[3]);
+            if (P.plan_is_log) {
+                v.x *= 0.6931471805599453f; v.y *= 0.6931471805599453f;
+                v.z *= 0.6931471805599453f; v.w *= 0.6931471805599453f;
+            } else {
+                v = make_float4(exp2f(v.x), exp2f(v.y), exp2f(v.z), exp2f(v.w));
+            }
+            float* const d = P.plan + (r0 + r) * P.ld_plan + c0 + c % M;
+            if (P.vec_plan) *reinterpret_cast<float4*>(d) = v;
+            else { d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w; }
+        }
+    }
+}
 
-template <int M, int MODE, int V>
-__global__ void __launch_bounds__(WARPS * 32, MinBlocks<M, V>::value) tsenor_kernel(const Params P) {
+template <class G, int MODE, bool EE> struct SmemLayout {   // of one warp
+    static constexpr int M = G::M;
+    // The score panel is kept beside the key panel for the local search, except that the whole
+    // method at M = 32 reads the scores of a block again when it needs them (RELOAD): the panel would
+    // cost the SM 4 of its 20 warps (14336 x 4096, 16:32: 3.13 ms with it, 3.03 without).
+    static constexpr bool RELOAD = (M == 32 && MODE == 0 && !EE);
+    static constexpr bool HAS_W = MODE != 1 && !RELOAD;
+    static constexpr int POT = (MODE == 2) ? 0 : 64 * (G::RO + G::CO);
+    static constexpr int CPRE = (M == 32 && MODE != 1) ? 32 * CPRE_STRIDE : 0;
+    static constexpr int AUX = (POT > CPRE) ? POT : CPRE;
+    alignas(16) float k[M * G::WS];     // scores, stash of t0, keys, row prefix tables in turn
+    float w[HAS_W ? M * G::WS : 1];
+    alignas(8) float aux[AUX ? AUX : 1];  // potentials, then the column-prefix tables of M = 32
+};
+// Resident warps per SM the register allocation aims for: 20 where the loop fits in 96 registers.
+template <int M, int V, bool EE> struct MinWarps { static constexpr int value = (M == 32 && !EE) ? 20 : 16; };
+// Warps per CTA.  One: 3 to 25 % faster than four on ragged widths (finer tail) and never slower,
+// with one exception.  The stopping test at M = 32 runs through the kernel's whole code for a dozen
+// iterations of work; four warps that go through it together (barriers after the loader and before
+// the rounding stage) share what they fetch of it (14336 x 4096: 0.90 ms apart, 0.71 together).
+template <int M, int V, bool EE> struct CtaWarps { static constexpr int value = (M == 32 && EE) ? 4 : 1; };
+
+// Cells of a lane's sub-tile in a shared-memory panel.
+template <class G> struct SubTile {
+    int r0, gr, c0, gc;
+    __device__ __forceinline__ explicit SubTile(int lane) {
+        using T = typename G::T;
+        const int g = lane % G::LPB, lr = g / T::PC, lc = g % T::PC;   // lane inside its block
+        r0 = lr * T::MR; gr = xor_perm<T::MR, T::PC>(lc);
+        c0 = lane / G::LPB * G::M + lc * T::MC; gc = xor_perm<T::MC, T::PR>(lr);
+    }
+    __device__ __forceinline__ int row(int a) const { return r0 + (a ^ gr); }
+    __device__ __forceinline__ int col(int b) const { return c0 + (b ^ gc); }
+};
+
+template <int M, int MODE, int V, bool EE>
+__global__ void __launch_bounds__(32 * CtaWarps<M, V, EE>::value, MinWarps<M, V, EE>::value / CtaWarps<M, V, EE>::value)
+tsenor_kernel(const Params P) {
     using G = Geom<M, V>;
     using T = typename G::T;
+    using L = SmemLayout<G, MODE, EE>;
     constexpr int MR = T::MR, MC = T::MC, PR = T::PR, PC = T::PC;
+    constexpr int WPC = CtaWarps<M, V, EE>::value;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    SmemLayout<G, MODE>& sm = *reinterpret_cast<SmemLayout<G, MODE>*>(smem_raw);
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t panel = blockIdx.x;
-    PanelMap<M> pm;
-    pm.tall = P.tall;
-    pm.rows = P.rows; pm.cols = P.cols;
+    const int lane = threadIdx.x % 32;
+    L& sm = reinterpret_cast<L*>(smem_raw)[threadIdx.x / 32];
 #ifdef TSENOR_BOUNDS
     if (threadIdx.x == 0) g_bounds_flags = 0;
     __syncthreads();
 #endif
-    if (P.tall) {
-        constexpr int NB = G::PANEL / M;
-        const int64_t left = P.rows / M - panel * NB;
-        pm.first = panel * NB; pm.r0 = 0; pm.c0 = 0;
-        pm.valid_cols = (int)(left < NB ? left : NB) * M;
-    } else {
-        pm.r0 = (panel / P.npc) * M;
-        pm.c0 = (panel % P.npc) * (int64_t)G::PANEL;
-        pm.first = 0;
-        pm.valid_cols = (int)((P.cols - pm.c0 < G::PANEL) ? (P.cols - pm.c0) : G::PANEL);
-    }
-    const int valid_cols = pm.valid_cols;
     int flags = 0;
 
     // ---- block loader
-    if (load_score_panel<G>(P.src, pm, sm.w)) flags |= DEV_NONFINITE;
-    if (MODE == 2)
-        if (load_key_panel<G>(P.keys, P.ld_keys, pm, P.vec_keys != 0, sm.k)) flags |= DEV_NONFINITE;
-    if (MODE != 1)
-        for (int idx = threadIdx.x; idx < M * G::WORDS; idx += WARPS * 32) sm.bits[idx] = 0u;
-    __syncthreads();
+    float* const panel = L::HAS_W ? sm.w : sm.k;
+    {
+        const UnitMap<M> um(P.rows, P.cols, P.nbp, this_unit<WPC>() * G::BPW);
+        if (load_scores<G, G::UW>(P.src, um, 0, lane, panel)) flags |= DEV_NONFINITE;
+        if (MODE == 2)
+            if (load_keys<G>(P.keys, P.ld_keys, um, P.vec_keys != 0, lane, sm.k)) flags |= DEV_NONFINITE;
+    }
+    if (WPC > 1) __syncthreads();
+    else __syncwarp();
 
     // ---- Algorithm 1
     if (MODE != 2) {
-        const int g = lane % G::LPB;                          // lane inside its block
-        const int blk = warp * G::BPW + lane / G::LPB;        // block inside the panel
-        const int lr = g / PC, lc = g % PC;
-        const int gr = xor_perm<MR, PC>(lc), gc = xor_perm<MC, PR>(lr);
-        const bool active = blk * M < valid_cols;
         float t[MR][MC];
         float mx[MR];
+        const SubTile<G> st0(lane);
 #pragma unroll
         for (int a = 0; a < MR; ++a) {
-            const int row = lr * MR + (a ^ gr);
             float m = 0.f;
 #pragma unroll
             for (int b = 0; b < MC; ++b) {
-                const int col = blk * M + lc * MC + (b ^ gc);
-                t[a][b] = TS_CHECK(row < M && col < G::PANEL) ? sm.w[row * G::WS + col] : 0.0f;
+                const int cell = st0.row(a) * G::WS + st0.col(b);
+                t[a][b] = TS_CHECK(st0.row(a) < M && st0.col(b) < G::UW) ? panel[cell] : 0.0f;
                 m = fmaxf(m, t[a][b]);
             }
             mx[a] = m;
@@ -942,6 +1093,7 @@ __global__ void __launch_bounds__(WARPS * 32, MinBlocks<M, V>::value) tsenor_ker
                 c_hi = 0.0f; c_lo = 0.0f;
             }
         }
+        __syncwarp();            // the score panel is read: its cells may become the stash
         if (P.iters > 0) {
 #pragma unroll
             for (int a = 0; a < MR; ++a) {
@@ -949,10 +1101,13 @@ __global__ void __launch_bounds__(WARPS * 32, MinBlocks<M, V>::value) tsenor_ker
 #pragma unroll
                 for (int b = 0; b < MC; ++b) t[a][b] = fmaf(t[a][b], c_lo, fmaf(t[a][b], c_hi, -sh));
             }
-            const int ran =
-                dykstra_iterate<G>(t, sm.k + warp * (32 * MR * MC), lane, P.Nf, P.log2N, P.iters, P.ee_eps);
+            const int ran = dykstra_iterate<G, EE>(t, sm.k, reinterpret_cast<float2*>(sm.aux), lane, P.Nf, P.log2N,
+                                                   P.iters, P.ee_eps);
             if (P.iter_sum) {   // one add per warp: iterations x blocks of the warp that exist
-                const int nact = __popc(__ballot_sync(FULL, active && g == 0));
+                const UnitMap<M> um(P.rows, P.cols, P.nbp, this_unit<WPC>() * G::BPW);
+                int64_t r0, c0;
+                const bool there = um.locate(lane / G::LPB, r0, c0);
+                const int nact = __popc(__ballot_sync(FULL, there && lane % G::LPB == 0));
                 if (lane == 0 && nact) atomicAdd(P.iter_sum, (unsigned long long)ran * nact);
             }
 #pragma unroll
@@ -965,65 +1120,52 @@ __global__ void __launch_bounds__(WARPS * 32, MinBlocks<M, V>::value) tsenor_ker
 #pragma unroll
                 for (int b = 0; b < MC; ++b) t[a][b] = fmaf(t[a][b], c_lo, t[a][b] * c_hi);
         }
-        if (MODE == 1) {
-            if (active) {
+        __syncwarp();            // sm.k served as stash until here; now it takes the keys
+        int l = lane;            // tied to the result of the iterations, so that the addresses of the
+        asm("" : "+r"(l), "+f"(t[0][0]));   // cells are worked out again and not kept over the loop
+        const SubTile<G> st(l);
 #pragma unroll
-                for (int a = 0; a < MR; ++a)
+        for (int a = 0; a < MR; ++a)
 #pragma unroll
-                    for (int b = 0; b < MC; ++b) {
-                        const int pc = blk * M + lc * MC + (b ^ gc);
-                        const int64_t row = pm.row(lr * MR + (a ^ gr), pc), col = pm.col(pc);
-                        if (TS_CHECK(row >= 0 && row < P.rows && col >= 0 && col < P.cols))
-                            P.plan[row * P.ld_plan + col] =
-                                P.plan_is_log ? t[a][b] * 0.6931471805599453f : exp2f(t[a][b]);
-                    }
-            }
-        } else {
-            __syncthreads();   // sm.k served as per-warp stash until here; now it takes the keys
-#pragma unroll
-            for (int a = 0; a < MR; ++a)
-#pragma unroll
-                for (int b = 0; b < MC; ++b)
-                    if (TS_CHECK(lr * MR + (a ^ gr) < M && blk * M + lc * MC + (b ^ gc) < G::PANEL))
-                        sm.k[(lr * MR + (a ^ gr)) * G::WS + blk * M + lc * MC + (b ^ gc)] = t[a][b];
-        }
+            for (int b = 0; b < MC; ++b)
+                if (TS_CHECK(st.row(a) < M && st.col(b) < G::UW)) sm.k[st.row(a) * G::WS + st.col(b)] = t[a][b];
         __syncwarp();
+        if (MODE == 1)           // ---- plan writer
+            store_plan<G>(P, UnitMap<M>(P.rows, P.cols, P.nbp, this_unit<WPC>() * G::BPW), lane, sm.k);
     }
 
-    // ---- Algorithm 2 and the mask writer
+    if (MODE == 0 && WPC > 1) __syncthreads();
+    // ---- Algorithm 2 and the mask writer: the blocks of one mask word (GPW M = 32 columns) a pass
     if (MODE != 1) {
-        const int grp = lane / M;
+        const int grp = lane / M, i = lane % M;
+        const auto unit_map = [&]() { return UnitMap<M>(P.rows, P.cols, P.nbp, this_unit<WPC>() * G::BPW); };
+        const UnitMap<M> um = unit_map();
 #pragma unroll 1
         for (int pass = 0; pass < G::PASSES; ++pass) {
-            const int blk = warp * G::BPW + pass * G::GPW + grp;
-            const bool active = (pass * G::GPW + grp < G::BPW) && blk * M < valid_cols;
-            if (!TS_CHECK(blk * M + M <= G::PANEL)) continue;     // warp-uniform up to the group
-            const unsigned row_bits =
-                round_block<G>(sm.k + blk * M, sm.w + blk * M, sm.cpre + (warp * 32 + lane) * CPRE_STRIDE, lane,
-                               active, P.N, P.ls_steps, flags);
-            if (active && TS_CHECK(blk * M / 32 < G::WORDS)) {
-                const int off = blk * M;
-                if (M == 32) sm.bits[(lane % M) * G::WORDS + off / 32] = row_bits;
-                else atomicOr(&sm.bits[(lane % M) * G::WORDS + off / 32], row_bits << (off % 32));
+            const int slot0 = pass * G::GPW, c = (slot0 + grp) * M;
+            int64_t r0, c0;
+            const bool active = um.locate(slot0 + grp, r0, c0);
+            if (!TS_CHECK(c + M <= G::UW)) continue;     // warp-uniform up to the group
+            const unsigned sel = round_block<G>(
+                sm.k + c, (L::RELOAD ? sm.k : sm.w) + c, reinterpret_cast<unsigned*>(sm.aux) + lane * CPRE_STRIDE,
+                lane, active, MODE == 0 && P.iters > 0, P.N, P.ls_steps, flags, [&]() {
+                    if (L::RELOAD) {
+                        __syncwarp();
+                        load_scores<G, 32>(P.src, unit_map(), slot0, lane, sm.k + slot0 * M);
+                        __syncwarp();
+                    }
+                });
+            if (M == 32) unit_map().locate(slot0 + grp, r0, c0);   // worked out again: one pass, few registers
+            if (P.nbp == 1) {       // a word for every row of every block
+                if (active && TS_CHECK(r0 + i < P.rows)) P.bits[(r0 + i) * P.wpr] = sel;
+            } else {                // the blocks of the pass share the words of their M rows
+                unsigned word = sel << (grp * M % 32);
+#pragma unroll
+                for (int s = M; s < 32; s <<= 1) word |= __shfl_xor_sync(FULL, word, s);
+                if (grp == 0 && active && TS_CHECK(r0 + i < P.rows && c0 / 32 < P.wpr))
+                    P.bits[(r0 + i) * P.wpr + c0 / 32] = word;
             }
             __syncwarp();
-        }
-        __syncthreads();
-        if (P.tall) {   // one word (M bits) per matrix row
-            constexpr unsigned GM = (M == 32) ? 0xffffffffu : ((1u << (M & 31)) - 1u);
-            for (int idx = threadIdx.x; idx < valid_cols; idx += WARPS * 32) {
-                const int blk = idx / M, r = idx % M;
-                if (TS_CHECK((pm.first + blk) * M + r < P.rows && (blk * M) / 32 < G::WORDS))
-                    P.bits[((pm.first + blk) * M + r) * P.wpr] =
-                        (sm.bits[r * G::WORDS + (blk * M) / 32] >> ((blk * M) % 32)) & GM;
-            }
-        } else {
-            const int nwords = (valid_cols + 31) / 32;
-            for (int idx = threadIdx.x; idx < M * G::WORDS; idx += WARPS * 32) {
-                const int r = idx / G::WORDS, wd = idx % G::WORDS;
-                if (wd < nwords && TS_CHECK(pm.r0 + r < P.rows && pm.c0 / 32 + wd < P.wpr))
-                    P.bits[(pm.r0 + r) * P.wpr + pm.c0 / 32 + wd] = sm.bits[idx];
-            }
         }
     }
 #ifdef TSENOR_BOUNDS

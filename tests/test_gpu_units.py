@@ -1,0 +1,63 @@
+"""Units of consecutive blocks: where a warp's blocks run on into the next block row, where a block
+row is padded to whole mask words, and where the scores are read again for the local search."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2505_23949_b200 import binding as ts
+from paper_2505_23949_b200 import synth
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(autouse=True, params=["throughput", "latency"])
+def _both_register_layouts(request):
+    ts.set_layout(ts.LAYOUT_THROUGHPUT if request.param == "throughput" else ts.LAYOUT_LATENCY)
+    yield
+    ts.set_layout(ts.LAYOUT_AUTO)
+
+
+# blocks per block row: one (a slab), fewer than share a mask word, one more than a word or a unit holds
+@pytest.mark.parametrize("nbc,nbr", [(1, 37), (2, 19), (3, 7), (5, 5), (9, 3), (17, 2), (33, 1)])
+@pytest.mark.parametrize("M,N", [(4, 1), (8, 3), (16, 8), (32, 16)])
+@pytest.mark.parametrize("pad", [0, 4, 5])
+def test_units_that_run_over_block_rows(M, N, nbc, nbr, pad):
+    rows, cols = nbr * M, nbc * M
+    W = synth.student_t_abs(rows, cols, 0.02, seed=nbc * 100 + M)
+    big = torch.zeros((rows, cols + pad), device=DEV)
+    big[:, pad:] = torch.from_numpy(W)
+    Wd = big[:, pad:]                       # rows start at an aligned address or not
+    tau = synth.default_tau(float(W.max()))
+    st = ts.new_status(DEV)
+    out = torch.full((rows, cols + pad), 7.0, device=DEV)
+    plan = ts.dykstra(Wd, N, M, tau, 60, plan_is_log=True, plan_out=out[:, pad:], status=st)
+    ref = oracle.dykstra(W, N, M, tau, 60)
+    # the plan's parity bound: fp32 rounding of t0 (ulp(288) in base-2 units) and of the potentials
+    assert np.abs(np.exp(plan.cpu().numpy().astype(np.float64)) - ref).max() <= 1e-4
+    assert bool((out[:, :pad] == 7.0).all())
+    mask = ts.new_mask(rows, cols, DEV).fill_(-1)
+    ts.solve(Wd, N, M, tau, 60, mask_out=mask, status=st)
+    keys = plan.cpu().numpy()
+    got = ts.round_plan(plan, Wd, N, M, status=st).cpu().numpy().view(np.uint32)
+    assert np.array_equal(got, oracle.round_plan(keys, W, N, M))      # rounding: bit for bit
+    # the fused kernel rounds the same plan in base-2 units, a positive multiple of the keys
+    # (products by ln 2 that round to equal keys are the only way to differ: none at these sizes)
+    assert np.array_equal(mask.cpu().numpy().view(np.uint32), got)
+    assert int(ts.check(mask, rows, cols, N, M).item()) == 0
+    assert int(st.item()) == 0
+
+
+@pytest.mark.parametrize("M", [4, 8, 16, 32])
+def test_keys_that_share_their_leading_bits(M):
+    """Lines whose keys differ only in the bits the packed sort words drop, in runs of every length."""
+    rng = np.random.default_rng(M)
+    rows, cols = 8 * M, 8 * M
+    base = rng.choice(np.array([-1.5, -0.75, 0.0, 0.5, 3.0], np.float32), size=(rows, cols))
+    bits = base.view(np.uint32) + np.where(base == 0, 0, rng.integers(0, 40, size=base.shape)).astype(np.uint32)
+    keys = bits.astype(np.uint32).view(np.float32)
+    W = synth.gaussian_abs(rows, cols, 0.02, seed=M)
+    for N in (1, M // 2):
+        got = ts.round_plan(torch.from_numpy(keys).to(DEV), torch.from_numpy(W).to(DEV), N, M)
+        assert np.array_equal(got.cpu().numpy().view(np.uint32), oracle.round_plan(keys, W, N, M))
