@@ -174,15 +174,32 @@ __global__ void fill_mask_kernel(uint32_t* bits, int64_t rows, int64_t wpr, int6
     }
 }
 
+// Walk over the quads (4 columns) of a matrix: quad idx is (row(idx), 4 * (idx - row(idx) * qpr)).
+// Rows by a multiplication with ceil(2^64 / qpr), exact while the quads number less than 2^32 (the
+// error of the quotient is then below idx / 2^64 < 1 / qpr); instead of a 64-bit division, some 100 instructions.
+struct QuadWalk {
+    int64_t qpr, nq;
+    unsigned long long magic;     // 0: divide
+    __device__ __forceinline__ int64_t row(int64_t idx) const {
+        return magic ? (int64_t)__umul64hi((unsigned long long)idx, magic) : idx / qpr;
+    }
+};
+QuadWalk quad_walk(int64_t rows, int64_t cols) {
+    QuadWalk q;
+    q.qpr = cols / 4;
+    q.nq = rows * q.qpr;
+    q.magic = (q.qpr > 1 && q.nq < (1LL << 32)) ? ~0ULL / (unsigned long long)q.qpr + 1 : 0;
+    return q;
+}
+
 // Retained score of up to two masks under one score source (quads of 4 columns).
 __global__ void objective_kernel(const tsenor::ScoreSrc S, const uint32_t* __restrict__ bits_a,
-                                 const uint32_t* __restrict__ bits_b, int64_t rows, int64_t cols, int64_t wpr,
-                                 double* out) {
+                                 const uint32_t* __restrict__ bits_b, const QuadWalk q, int64_t wpr, double* out) {
     double acc_a = 0.0, acc_b = 0.0;
-    const int64_t qpr = cols / 4, nq = rows * qpr;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < nq;
+    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < q.nq;
          idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = idx / qpr, c = (idx % qpr) * 4;
+        // (the division overlaps the fp64 adds here: 12 us for a 2048 x 2048 matrix with it, 13.5 with q.row)
+        const int64_t r = idx / q.qpr, c = (idx % q.qpr) * 4;
         const uint32_t ma = (bits_a[r * wpr + c / 32] >> (c % 32)) & 15u;
         const uint32_t mb = bits_b ? (bits_b[r * wpr + c / 32] >> (c % 32)) & 15u : 0u;
         if ((ma | mb) == 0u) continue;
@@ -225,82 +242,35 @@ __global__ void keep_better_kernel(const double* __restrict__ obj2, const uint32
         mask_inout[idx] = prev[idx];
 }
 
-__global__ void scores_max_kernel(const tsenor::ScoreSrc S, int64_t rows, int64_t cols, unsigned int* out_bits) {
+// One atomic per CTA: with one per warp, 19,000 of them queued on a single word were two thirds of the
+// time (2048 x 2048: 16.4 us, 8.4 now; 4096 x 4096: 21.8 and 16.5).
+__global__ void scores_max_kernel(const tsenor::ScoreSrc S, const QuadWalk q, unsigned int* out_bits) {
     float m = 0.f;
-    const int64_t qpr = cols / 4, nq = rows * qpr;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < nq;
+    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < q.nq;
          idx += (int64_t)gridDim.x * blockDim.x) {
-        const float4 v = tsenor::load_score_quad(S, idx / qpr, (idx % qpr) * 4);
+        const int64_t r = q.row(idx);
+        const float4 v = tsenor::load_score_quad(S, r, (idx - r * q.qpr) * 4);
         m = fmaxf(fmaxf(m, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));  // fmaxf drops NaN
     }
-    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     // non-negative floats order like their bit patterns
-    if ((threadIdx.x & 31) == 0) atomicMax(out_bits, __float_as_uint(m));
+    const unsigned warp_max = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+    __shared__ unsigned part[32];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = warp_max;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const unsigned p = (threadIdx.x < (blockDim.x >> 5)) ? part[threadIdx.x] : 0u;
+        const unsigned cta_max = __reduce_max_sync(0xffffffffu, p);
+        if (threadIdx.x == 0) atomicMax(out_bits, cta_max);
+    }
 }
 
-__global__ void materialize_kernel(const tsenor::ScoreSrc S, int64_t rows, int64_t cols, float* out,
-                                   int64_t ld_out) {
-    const int64_t qpr = cols / 4, nq = rows * qpr;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < nq;
+__global__ void materialize_kernel(const tsenor::ScoreSrc S, const QuadWalk q, float* out, int64_t ld_out) {
+    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < q.nq;
          idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = idx / qpr, c = (idx % qpr) * 4;
+        const int64_t r = q.row(idx), c = (idx - r * q.qpr) * 4;
         const float4 v = tsenor::load_score_quad(S, r, c);
         float* p = out + r * ld_out + c;
         p[0] = v.x; p[1] = v.y; p[2] = v.z; p[3] = v.w;
-    }
-}
-
-// "Simple" rounding: one warp per block; lane i is row i in the first pass and column i in
-// the second.  Ranks by counting under the strict order (key descending, index ascending).
-__device__ __forceinline__ bool key_before(float ka, int ia, float kb, int ib) {
-    return ka > kb || (ka == kb && ia < ib);
-}
-__global__ void simple_round_kernel(const float* __restrict__ key, int64_t ld, int64_t rows, int64_t cols,
-                                    int64_t wpr, int N, int M, uint32_t* bits) {
-    __shared__ float ks[4][32][33];
-    __shared__ unsigned rowmask[4][32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t nbc = cols / M, nblk = (rows / M) * nbc;
-    for (int64_t b = blockIdx.x * 4LL + warp; b < nblk; b += gridDim.x * 4LL) {
-        const int64_t r0 = (b / nbc) * M, c0 = (b % nbc) * M;
-        for (int i = 0; i < M; ++i)
-            if (lane < M) {
-                float k = key[(r0 + i) * ld + c0 + lane];
-                if (!(k == k)) k = __int_as_float(0xff800000);
-                ks[warp][i][lane] = k + 0.0f;
-            }
-        __syncwarp();
-        unsigned keep = 0u;
-        if (lane < M) {   // row pass: the N best of my row
-            for (int j = 0; j < M; ++j) {
-                int rank = 0;
-                for (int j2 = 0; j2 < M; ++j2) rank += key_before(ks[warp][lane][j2], j2, ks[warp][lane][j], j) ? 1 : 0;
-                if (rank < N) keep |= 1u << j;
-            }
-        }
-        rowmask[warp][lane] = keep;
-        __syncwarp();
-        unsigned colkeep = 0u;   // bits over rows, for my column
-        if (lane < M) {
-            unsigned surv = 0u;
-            for (int i = 0; i < M; ++i) surv |= ((rowmask[warp][i] >> lane) & 1u) << i;
-            for (int i = 0; i < M; ++i) {
-                if (!((surv >> i) & 1u)) continue;
-                int rank = 0;
-                for (int i2 = 0; i2 < M; ++i2)
-                    if ((surv >> i2) & 1u) rank += key_before(ks[warp][i2][lane], i2, ks[warp][i][lane], i) ? 1 : 0;
-                if (rank < N) colkeep |= 1u << i;
-            }
-        }
-        __syncwarp();
-        rowmask[warp][lane] = colkeep;   // now indexed by column
-        __syncwarp();
-        if (lane < M) {
-            unsigned row = 0u;
-            for (int j = 0; j < M; ++j) row |= ((rowmask[warp][j] >> lane) & 1u) << j;
-            if (row) atomicOr(&bits[(r0 + lane) * wpr + c0 / 32], row << (c0 % 32));
-        }
-        __syncwarp();
     }
 }
 
@@ -341,6 +311,34 @@ int grid_for(int64_t work, int threads) {
     if (g < 1) g = 1;
     if (g > 148 * 16) g = 148 * 16;
     return (int)g;
+}
+
+// CTAs of 256 threads for the maximum over quads: one wave of full SMs, since every CTA ends in an atomic.
+int scan_grid(int64_t quads) {
+    const int64_t g = (quads + 255) / 256, wave = 8LL * sm_count();
+    return (int)(g < 1 ? 1 : g < wave ? g : wave);
+}
+
+// CTAs of 512 threads for the objectives: two waves (the fp64 sums make the CTAs uneven), and half the
+// atomics on one word that CTAs of 256 threads end in (safeguard of a 1024 x 1024 matrix: 10.6 -> 8.5 us).
+int objective_grid(int64_t quads) {
+    const int64_t g = (quads + 511) / 512, waves = 8LL * sm_count();
+    return (int)(g < 1 ? 1 : g < waves ? g : waves);
+}
+
+// Simple rounding, on the units of the rounding stage that are one mask word wide.
+template <int M>
+int launch_simple_round(const float* key, int64_t ld, int64_t rows, int64_t cols, int N, uint32_t* bits,
+                        cudaStream_t st) {
+    tsenor::Params P{};
+    P.rows = rows; P.cols = cols;
+    int64_t nbp = 0;
+    const int64_t units = unit_count<M, (M < 32) ? 1 : 0>(P, &nbp);
+    const int64_t ctas = (units + tsenor::SIMPLE_WARPS - 1) / tsenor::SIMPLE_WARPS;
+    if (ctas > 0x7fffffffLL) return TSENOR_ERR_SHAPE;
+    tsenor::simple_round_kernel<M><<<(unsigned)ctas, 32 * tsenor::SIMPLE_WARPS, 0, st>>>(
+        key, ld, rows, cols, (cols + 31) / 32, nbp, units, aligned16(key, ld), N, bits);
+    return finish_launch();
 }
 
 int trivial_mask(uint32_t* bits, int64_t rows, int64_t cols, bool ones, cudaStream_t st) {
@@ -414,8 +412,8 @@ int tsenor_solve_scores(const tsenor_scores_t* s, int64_t rows, int64_t cols, in
 static int max_on(const tsenor::ScoreSrc& src, int64_t rows, int64_t cols, float* dev_max_out, cudaStream_t st) {
     if (cudaMemsetAsync(dev_max_out, 0, sizeof(float), st) != cudaSuccess) return finish_launch(), TSENOR_ERR_CUDA;
     if (rows == 0 || cols == 0) return TSENOR_OK;
-    scores_max_kernel<<<grid_for(rows * (cols / 4), 256 * 2), 256, 0, st>>>(
-        src, rows, cols, reinterpret_cast<unsigned int*>(dev_max_out));
+    scores_max_kernel<<<scan_grid(rows * (cols / 4)), 256, 0, st>>>(src, quad_walk(rows, cols),
+                                                                    reinterpret_cast<unsigned int*>(dev_max_out));
     return finish_launch();
 }
 
@@ -435,8 +433,8 @@ int tsenor_scores_materialize(const tsenor_scores_t* s, int64_t rows, int64_t co
     if (int rc = make_source(s, cols, &src)) return rc;
     if (rows == 0 || cols == 0) return TSENOR_OK;
     if (!scores_out) return TSENOR_ERR_NULL;
-    materialize_kernel<<<grid_for(rows * (cols / 4), 256), 256, 0, (cudaStream_t)stream>>>(src, rows, cols,
-                                                                                          scores_out, ld_out);
+    materialize_kernel<<<grid_for(rows * (cols / 4), 256), 256, 0, (cudaStream_t)stream>>>(
+        src, quad_walk(rows, cols), scores_out, ld_out);
     return finish_launch();
 }
 
@@ -452,8 +450,8 @@ int tsenor_keep_better(const tsenor_scores_t* s, int64_t rows, int64_t cols, con
     if (rows == 0 || cols == 0) return TSENOR_OK;
     if (!prev_mask || !mask_inout) return TSENOR_ERR_NULL;
     const int64_t wpr = (cols + 31) / 32;
-    objective_kernel<<<grid_for(rows * (cols / 4), 256), 256, 0, st>>>(src, mask_inout, prev_mask, rows, cols, wpr,
-                                                                      dev_obj2_out);
+    objective_kernel<<<objective_grid(rows * (cols / 4)), 512, 0, st>>>(src, mask_inout, prev_mask, quad_walk(rows, cols),
+                                                                   wpr, dev_obj2_out);
     if (int rc = finish_launch()) return rc;
     keep_better_kernel<<<grid_for(rows * wpr, 256), 256, 0, st>>>(dev_obj2_out, prev_mask, mask_inout, rows * wpr);
     return finish_launch();
@@ -466,11 +464,12 @@ int tsenor_simple_round(const float* plan_key, int64_t ld_plan, int64_t rows, in
     if (rows == 0 || cols == 0) return TSENOR_OK;
     if (!plan_key || !mask_bits_out) return TSENOR_ERR_NULL;
     cudaStream_t st = (cudaStream_t)stream;
-    const int64_t wpr = (cols + 31) / 32, nblk = (rows / M) * (cols / M);
-    if (cudaMemsetAsync(mask_bits_out, 0, sizeof(uint32_t) * (size_t)(rows * wpr), st) != cudaSuccess)
-        return finish_launch(), TSENOR_ERR_CUDA;
-    simple_round_kernel<<<grid_for(nblk, 4), 128, 0, st>>>(plan_key, ld_plan, rows, cols, wpr, N, M, mask_bits_out);
-    return finish_launch();
+    switch (M) {
+        case 4: return launch_simple_round<4>(plan_key, ld_plan, rows, cols, N, mask_bits_out, st);
+        case 8: return launch_simple_round<8>(plan_key, ld_plan, rows, cols, N, mask_bits_out, st);
+        case 16: return launch_simple_round<16>(plan_key, ld_plan, rows, cols, N, mask_bits_out, st);
+        default: return launch_simple_round<32>(plan_key, ld_plan, rows, cols, N, mask_bits_out, st);
+    }
 }
 
 static int dykstra_on(const tsenor::ScoreSrc& src, const Extras& x, int64_t rows, int64_t cols, int N, int M,
@@ -550,8 +549,8 @@ int tsenor_objective(const float* scores, int64_t ld, const uint32_t* mask_bits,
     if (rows == 0 || cols == 0) return TSENOR_OK;
     if (!scores || !mask_bits) return TSENOR_ERR_NULL;
     const int64_t wpr = (cols + 31) / 32;
-    objective_kernel<<<grid_for(rows * (cols / 4), 256), 256, 0, st>>>(abs_source(scores, ld), mask_bits, nullptr,
-                                                                      rows, cols, wpr, dev_sum_out);
+    objective_kernel<<<objective_grid(rows * (cols / 4)), 512, 0, st>>>(abs_source(scores, ld), mask_bits, nullptr,
+                                                                   quad_walk(rows, cols), wpr, dev_sum_out);
     return finish_launch();
 }
 

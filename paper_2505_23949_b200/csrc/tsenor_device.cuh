@@ -458,39 +458,41 @@ __device__ __forceinline__ float score_of(int kind, float w, float v, float scal
     }
 }
 
-// Scores of the four consecutive elements (r, c .. c+3); c is a multiple of 4.
-__device__ __forceinline__ float4 load_score_quad(const ScoreSrc& S, int64_t r, int64_t c) {
-    float4 w;
-    if (S.w_is_bf16) {
-        const unsigned short* p = static_cast<const unsigned short*>(S.w) + r * S.ld + c;
-        unsigned lo, hi;
-        if (S.vec_w) {
-            const uint2 q = __ldg(reinterpret_cast<const uint2*>(p));
-            lo = q.x; hi = q.y;
-        } else {
-            lo = __ldg(p) | ((unsigned)__ldg(p + 1) << 16);
-            hi = __ldg(p + 2) | ((unsigned)__ldg(p + 3) << 16);
-        }
-        w = make_float4(__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u),
-                        __uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
-    } else {
-        const float* p = static_cast<const float*>(S.w) + r * S.ld + c;
-        if (S.vec_w) w = __ldg(reinterpret_cast<const float4*>(p));
-        else w = make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+__device__ __forceinline__ float4 widen_bf16(unsigned lo, unsigned hi) {
+    return make_float4(__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u),
+                       __uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+}
+__device__ __forceinline__ float4 load_float_quad(const float* p, bool vec) {
+    return vec ? __ldg(reinterpret_cast<const float4*>(p))
+               : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+}
+// Weights of the four consecutive elements (r, c .. c+3); c is a multiple of 4.
+__device__ __forceinline__ float4 load_weight_quad(const ScoreSrc& S, int64_t r, int64_t c) {
+    if (!S.w_is_bf16) return load_float_quad(static_cast<const float*>(S.w) + r * S.ld + c, S.vec_w != 0);
+    const unsigned short* p = static_cast<const unsigned short*>(S.w) + r * S.ld + c;
+    if (S.vec_w) {
+        const uint2 q = __ldg(reinterpret_cast<const uint2*>(p));
+        return widen_bf16(q.x, q.y);
     }
+    return widen_bf16(__ldg(p) | ((unsigned)__ldg(p + 1) << 16), __ldg(p + 2) | ((unsigned)__ldg(p + 3) << 16));
+}
+// Entries c .. c+3 of the column vector (ones for the kinds without one).
+__device__ __forceinline__ float4 load_colvec_quad(const ScoreSrc& S, int64_t c) {
+    return (S.kind >= SC_COLDIV) ? load_float_quad(S.colvec + c, S.vec_c != 0) : make_float4(1.f, 1.f, 1.f, 1.f);
+}
+// Scores of the four consecutive elements (r, c .. c+3); colvec(c) gives their column-vector entries.
+template <class Colvec>
+__device__ __forceinline__ float4 load_score_quad(const ScoreSrc& S, int64_t r, int64_t c, Colvec colvec) {
+    const float4 w = load_weight_quad(S, r, c);
     if (S.kind == SC_ABS) return make_float4(fabsf(w.x), fabsf(w.y), fabsf(w.z), fabsf(w.w));
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f), cv = make_float4(1.f, 1.f, 1.f, 1.f);
-    if (S.kind == SC_ADMM) {
-        const float* p = S.v + r * S.ld_v + c;
-        if (S.vec_v) v = __ldg(reinterpret_cast<const float4*>(p));
-        else v = make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
-    } else {
-        const float* p = S.colvec + c;
-        if (S.vec_c) cv = __ldg(reinterpret_cast<const float4*>(p));
-        else cv = make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
-    }
+    const float4 cv = colvec(c);
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (S.kind == SC_ADMM) v = load_float_quad(S.v + r * S.ld_v + c, S.vec_v != 0);
     return make_float4(score_of(S.kind, w.x, v.x, S.scalar, cv.x), score_of(S.kind, w.y, v.y, S.scalar, cv.y),
                        score_of(S.kind, w.z, v.z, S.scalar, cv.z), score_of(S.kind, w.w, v.w, S.scalar, cv.w));
+}
+__device__ __forceinline__ float4 load_score_quad(const ScoreSrc& S, int64_t r, int64_t c) {
+    return load_score_quad(S, r, c, [&](int64_t col) { return load_colvec_quad(S, col); });
 }
 
 __device__ __forceinline__ int any_nan(const float4& v) {
@@ -546,15 +548,15 @@ template <int M> struct UnitMap {
 // ---------------------------------------------------------------------------
 // Unit loaders: COLS columns (from slot `slot0` on) of the unit's M rows into shared memory
 // (dst: row stride WS), coalesced, vector loads when the addresses allow it.  A lane keeps its
-// column(s) and walks down the rows, BATCH of them in flight: the position is worked out once.
-// The common source (fp32 |W|, aligned) has a loop of its own with every load in flight; the
-// others share one that is unrolled less, because the instruction cache is what the warps of
-// an SM, spread over all phases of the kernel, compete for.  Return non-zero if this lane saw a
-// non-finite score, respectively a NaN key.
+// column(s) and walks down the rows, BATCH of them in flight: the position, and the entries of the
+// column vector, are worked out once.  Aligned sources have loops of their own with many
+// loads in flight; the others share one that is unrolled less, because the instruction cache is
+// what the warps of an SM, spread over all phases of the kernel, compete for.  Return non-zero if
+// this lane saw a non-finite score, respectively a NaN key.
 // ---------------------------------------------------------------------------
-template <class G, int COLS, int BATCH, class Load>
+template <class G, int COLS, int BATCH, class Column, class Load>
 __device__ __forceinline__ void load_unit(const UnitMap<G::M>& um, int slot0, int lane, float* __restrict__ dst,
-                                          Load load) {
+                                          Column column, Load load) {
     constexpr int M = G::M;
     constexpr int QW = (COLS / 4 < 32) ? COLS / 4 : 32;     // quads of a row that the warp takes at once
     constexpr int RPI = 32 / QW, STEPS = M / RPI;           // rows it takes at once
@@ -568,6 +570,7 @@ __device__ __forceinline__ void load_unit(const UnitMap<G::M>& um, int slot0, in
         r0 += lane / QW;
         c0 += c % M;
         float* d = dst + (lane / QW) * G::WS + c;
+        if (there) column(c0);
 #pragma unroll 1
         for (int i0 = 0; i0 < STEPS; i0 += B, r0 += B * RPI, d += B * RPI * G::WS) {
             float4 v[B];
@@ -593,15 +596,45 @@ __device__ __forceinline__ int load_scores(const ScoreSrc& S, const UnitMap<G::M
         nan = fmaf(v.x, 0.0f, fmaf(v.y, 0.0f, fmaf(v.z, 0.0f, fmaf(v.w, 0.0f, nan))));
         return v;
     };
+    float4 cv = make_float4(1.f, 1.f, 1.f, 1.f);
+    const auto no_column = [](int64_t) {};
+    const auto column = [&](int64_t c) { cv = load_colvec_quad(S, c); };
+    const auto scaled = [&](const float4& v) {      // |w| 1 is |w|
+        return seen(make_float4(__fmul_rn(fabsf(v.x), cv.x), __fmul_rn(fabsf(v.y), cv.y),
+                                __fmul_rn(fabsf(v.z), cv.z), __fmul_rn(fabsf(v.w), cv.w)));
+    };
+    const float* const w32 = static_cast<const float*>(S.w);
+    const unsigned short* const w16 = static_cast<const unsigned short*>(S.w);
     if (S.kind == SC_ABS && !S.w_is_bf16 && S.vec_w) {
-        const float* const w = static_cast<const float*>(S.w);
-        load_unit<G, COLS, 8>(um, slot0, lane, dst, [&](int64_t r, int64_t c) {
-            const float4 v = __ldg(reinterpret_cast<const float4*>(w + r * S.ld + c));
+        load_unit<G, COLS, 8>(um, slot0, lane, dst, no_column, [&](int64_t r, int64_t c) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(w32 + r * S.ld + c));
             return seen(make_float4(fabsf(v.x), fabsf(v.y), fabsf(v.z), fabsf(v.w)));
         });
+    } else if ((S.kind == SC_ABS || S.kind == SC_COLMUL) && S.vec_w && S.w_is_bf16) {
+        load_unit<G, COLS, 8>(um, slot0, lane, dst, column, [&](int64_t r, int64_t c) {
+            const uint2 q = __ldg(reinterpret_cast<const uint2*>(w16 + r * S.ld + c));
+            return scaled(widen_bf16(q.x, q.y));
+        });
+    } else if (S.kind == SC_COLMUL && S.vec_w) {
+        load_unit<G, COLS, 4>(um, slot0, lane, dst, column, [&](int64_t r, int64_t c) {
+            return scaled(__ldg(reinterpret_cast<const float4*>(w32 + r * S.ld + c)));
+        });
+    } else if (S.kind == SC_ADMM && S.vec_w && S.vec_v && !S.w_is_bf16) {
+        load_unit<G, COLS, 4>(um, slot0, lane, dst, no_column, [&](int64_t r, int64_t c) {
+            const float4 w = __ldg(reinterpret_cast<const float4*>(w32 + r * S.ld + c));
+            const float4 v = __ldg(reinterpret_cast<const float4*>(S.v + r * S.ld_v + c));
+            return seen(make_float4(score_of(SC_ADMM, w.x, v.x, S.scalar, 1.f), score_of(SC_ADMM, w.y, v.y, S.scalar, 1.f),
+                                    score_of(SC_ADMM, w.z, v.z, S.scalar, 1.f), score_of(SC_ADMM, w.w, v.w, S.scalar, 1.f)));
+        });
+    } else if (S.kind == SC_COLDIV && S.vec_w && !S.w_is_bf16) {
+        load_unit<G, COLS, 4>(um, slot0, lane, dst, column, [&](int64_t r, int64_t c) {
+            const float4 w = __ldg(reinterpret_cast<const float4*>(w32 + r * S.ld + c));
+            return seen(make_float4(fabsf(__fdiv_rn(w.x, cv.x)), fabsf(__fdiv_rn(w.y, cv.y)),
+                                    fabsf(__fdiv_rn(w.z, cv.z)), fabsf(__fdiv_rn(w.w, cv.w))));
+        });
     } else {
-        load_unit<G, COLS, 2>(um, slot0, lane, dst,
-                              [&](int64_t r, int64_t c) { return seen(load_score_quad(S, r, c)); });
+        load_unit<G, COLS, 2>(um, slot0, lane, dst, column,
+                              [&](int64_t r, int64_t c) { return seen(load_score_quad(S, r, c, [&](int64_t) { return cv; })); });
     }
     return nan != 0.0f;
 }
@@ -609,10 +642,8 @@ template <class G>
 __device__ __forceinline__ int load_keys(const float* __restrict__ src, int64_t ld, const UnitMap<G::M>& um,
                                          bool vec_ok, int lane, float* __restrict__ dst) {
     int bad = 0;
-    load_unit<G, G::UW, 4>(um, 0, lane, dst, [&](int64_t r, int64_t c) {
-        const float* p = src + r * ld + c;
-        const float4 v = vec_ok ? __ldg(reinterpret_cast<const float4*>(p))
-                                : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+    load_unit<G, G::UW, 4>(um, 0, lane, dst, [](int64_t) {}, [&](int64_t r, int64_t c) {
+        const float4 v = load_float_quad(src + r * ld + c, vec_ok);
         bad |= any_nan(v);          // infinite keys have a place in the order; NaN keys are flagged
         return v;
     });
@@ -947,6 +978,72 @@ __device__ __forceinline__ unsigned round_block(float* ks, const float* ws, unsi
     return sel;
 }
 
+// The mask rows of the (up to) 32 / M blocks a warp has just rounded: lane i of group grp holds
+// row i of the block at (r0, c0).  In a slab every block's rows have words of their own; else the
+// blocks share the words of their M rows.
+template <int M>
+__device__ __forceinline__ void write_mask_rows(uint32_t* bits, int64_t wpr, int64_t rows, int64_t nbp, int64_t r0,
+                                                int64_t c0, int lane, bool active, unsigned sel) {
+    const int grp = lane / M, i = lane % M;
+    if (nbp == 1) {
+        if (active && TS_CHECK(r0 + i < rows)) bits[(r0 + i) * wpr] = sel;
+        return;
+    }
+    unsigned word = sel << (grp * M % 32);
+#pragma unroll
+    for (int s = M; s < 32; s <<= 1) word |= __shfl_xor_sync(FULL, word, s);
+    if (grp == 0 && active && TS_CHECK(r0 + i < rows && c0 / 32 < wpr)) bits[(r0 + i) * wpr + c0 / 32] = word;
+}
+
+// ---------------------------------------------------------------------------
+// "Simple" rounding (Appendix B.2): the N best keys of every row, then the N best survivors of
+// every column.  A warp takes one mask word's width of blocks, a lane one row and one column, and
+// both passes are read off the sorted order of the line (the same networks as the greedy
+// selection's).  Bound by the ALU work of the sorts.  2048 x 2048, 8:16: 112 us for ranks by counting
+// (M compares per key, from shared memory), 16 us this way.
+// ---------------------------------------------------------------------------
+constexpr int SIMPLE_WARPS = 4;   // per CTA; independent of one another
+template <int M>
+__global__ void __launch_bounds__(32 * SIMPLE_WARPS)
+simple_round_kernel(const float* __restrict__ key, int64_t ld, int64_t rows, int64_t cols, int64_t wpr, int64_t nbp,
+                    int64_t units, int vec, int N, uint32_t* bits) {
+    using G = Geom<M, (M < 32) ? 1 : 0>;
+    static_assert(G::UW == 32 && G::PASSES == 1, "one mask word wide");
+    __shared__ float ks[SIMPLE_WARPS][M * G::WS];
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, i = lane % M;
+    const int64_t unit = (int64_t)blockIdx.x * SIMPLE_WARPS + warp;
+    if (unit >= units) return;
+    const UnitMap<M> um(rows, cols, nbp, unit * G::BPW);
+    load_keys<G>(key, ld, um, vec != 0, lane, ks[warp]);
+    __syncwarp();
+    const float* const blk = ks[warp] + lane / M * M;
+    unsigned kept = 0u;              // row pass: my row's columns; column pass: my column's rows
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+        const float* const line = side ? blk + i : blk + i * G::WS;
+        const int st = side ? G::WS : 1;
+        float k[M];
+        unsigned w[M];
+#pragma unroll
+        for (int j = 0; j < M; ++j) k[j] = line[j * st];
+        sort_line<M>(k, line, st, false, w);
+        const unsigned avail = side ? transpose_bits<M>(kept, i) : 0xffffffffu;
+        int left = N;
+        kept = 0u;
+#pragma unroll
+        for (int p = 0; p < M; ++p) {
+            const unsigned bit = 1u << (w[p] & 31u);
+            const bool take = left > 0 && (avail & bit) != 0u;
+            kept |= take ? bit : 0u;
+            left -= take ? 1 : 0;
+        }
+    }
+    int64_t r0, c0;
+    const bool active = um.locate(lane / M, r0, c0);
+    const unsigned row = transpose_bits<M>(kept, i);
+    write_mask_rows<M>(bits, wpr, rows, nbp, r0, c0, lane, active, active ? row : 0u);
+}
+
 // ---------------------------------------------------------------------------
 // Fused kernel.  MODE 0: whole method; 1: Algorithm 1 only (plan to global);
 // 2: Algorithm 2 only (keys from global).
@@ -1137,7 +1234,7 @@ tsenor_kernel(const Params P) {
     if (MODE == 0 && WPC > 1) __syncthreads();
     // ---- Algorithm 2 and the mask writer: the blocks of one mask word (GPW M = 32 columns) a pass
     if (MODE != 1) {
-        const int grp = lane / M, i = lane % M;
+        const int grp = lane / M;
         const auto unit_map = [&]() { return UnitMap<M>(P.rows, P.cols, P.nbp, this_unit<WPC>() * G::BPW); };
         const UnitMap<M> um = unit_map();
 #pragma unroll 1
@@ -1156,15 +1253,7 @@ tsenor_kernel(const Params P) {
                     }
                 });
             if (M == 32) unit_map().locate(slot0 + grp, r0, c0);   // worked out again: one pass, few registers
-            if (P.nbp == 1) {       // a word for every row of every block
-                if (active && TS_CHECK(r0 + i < P.rows)) P.bits[(r0 + i) * P.wpr] = sel;
-            } else {                // the blocks of the pass share the words of their M rows
-                unsigned word = sel << (grp * M % 32);
-#pragma unroll
-                for (int s = M; s < 32; s <<= 1) word |= __shfl_xor_sync(FULL, word, s);
-                if (grp == 0 && active && TS_CHECK(r0 + i < P.rows && c0 / 32 < P.wpr))
-                    P.bits[(r0 + i) * P.wpr + c0 / 32] = word;
-            }
+            write_mask_rows<M>(P.bits, P.wpr, P.rows, P.nbp, r0, c0, lane, active, sel);
             __syncwarp();
         }
     }

@@ -61,3 +61,40 @@ def test_keys_that_share_their_leading_bits(M):
     for N in (1, M // 2):
         got = ts.round_plan(torch.from_numpy(keys).to(DEV), torch.from_numpy(W).to(DEV), N, M)
         assert np.array_equal(got.cpu().numpy().view(np.uint32), oracle.round_plan(keys, W, N, M))
+
+
+@pytest.mark.parametrize("nbc,nbr", [(1, 5), (3, 3), (9, 2)])
+@pytest.mark.parametrize("M,N", [(4, 3), (8, 1), (16, 5), (32, 31)])
+def test_simple_rounding_writes_every_word(M, N, nbc, nbr):
+    rows, cols = nbr * M, nbc * M
+    rng = np.random.default_rng(M + nbc)
+    keys = rng.choice(np.array([-np.inf, np.nan, -2.0, -0.0, 0.0, 1.0, np.inf], np.float32), size=(rows, cols))
+    mask = ts.new_mask(rows, cols, DEV).fill_(-1)
+    ts.simple_round(torch.from_numpy(keys).to(DEV), N, M, mask_out=mask)
+    want = oracle.simple_round(np.where(np.isnan(keys), -np.inf, keys).astype(np.float32), N, M)
+    assert np.array_equal(mask.cpu().numpy().view(np.uint32), want)
+
+
+@pytest.mark.parametrize("kind", ["abs", "mul", "div", "admm"])
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("pad", [0, 5])
+def test_every_loader_sees_the_same_scores(kind, bf16, pad):
+    """The unit loaders (one per aligned source, one for the rest) against the materialised scores."""
+    rows, cols, M, N = 64, 160, 32, 16
+    g = torch.Generator(device=DEV).manual_seed(5)
+    big = torch.randn((rows, cols + pad), generator=g, device=DEV)
+    w = (big.to(torch.bfloat16) if bf16 else big)[:, pad:]
+    v = torch.randn((rows, cols), generator=g, device=DEV)
+    a = torch.randn(cols, generator=g, device=DEV).abs_() + 0.1
+    src = {"abs": lambda: ts.Scores(ts.SCORES_ABS, w), "mul": lambda: ts.Scores(ts.SCORES_COLMUL, w, colvec=a),
+           "div": lambda: ts.Scores(ts.SCORES_COLDIV, w, colvec=a),
+           "admm": lambda: ts.Scores(ts.SCORES_ADMM, w, v=v, scalar=0.5)}[kind]()
+    plain = ts.scores_materialize(src)
+    tau = 200.0 / float(ts.scores_max(src).item())
+    assert float(plain.max().item()) == float(ts.scores_max(src).item())
+    assert torch.equal(ts.solve_scores(src, N, M, tau, 40), ts.solve(plain, N, M, tau, 40))
+    assert torch.equal(ts.dykstra_scores(src, N, M, tau, 40), ts.dykstra(plain, N, M, tau, 40))
+    w[rows // 2, 3] = float("nan")
+    st = ts.new_status(DEV)
+    ts.solve_scores(src, N, M, tau, 5, status=st)
+    assert int(st.item()) & ts.DEV_NONFINITE_SCORE
