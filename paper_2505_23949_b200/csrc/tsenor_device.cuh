@@ -788,15 +788,22 @@ template <int M> __device__ __forceinline__ unsigned prefix_at(const void* tab, 
 
 // The first `cap` entries of `avail` (a set of positions of one line) in the line's sorted
 // order, or all of them if there are no more than `cap`: binary search for the shortest
-// prefix of the order that holds `cap` available entries.
+// prefix of the order that holds `cap` available entries.  For the lane's row and its column at
+// once and without branches: the two searches are chains of dependent shared-memory reads, and a
+// round of the greedy selection waits for them.
 template <int M>
-__device__ __forceinline__ unsigned first_available(unsigned avail, int cap, const void* tab) {
-    if (__popc(avail) <= cap) return avail;
-    int p = 0;
+__device__ __forceinline__ void first_available(unsigned& setR, int capR, const void* tabR, unsigned& setC, int capC,
+                                                const void* tabC) {
+    int p = 0, q = 0;
 #pragma unroll
-    for (int b = M / 2; b > 0; b >>= 1)
-        if (__popc(avail & prefix_at<M>(tab, p + b - 1)) < cap) p += b;
-    return avail & prefix_at<M>(tab, p);
+    for (int b = M / 2; b > 0; b >>= 1) {
+        const unsigned r = prefix_at<M>(tabR, p + b - 1), c = prefix_at<M>(tabC, q + b - 1);
+        p += (__popc(setR & r) < capR) ? b : 0;
+        q += (__popc(setC & c) < capC) ? b : 0;
+    }
+    const unsigned r = prefix_at<M>(tabR, p), c = prefix_at<M>(tabC, q);
+    setR &= (__popc(setR) <= capR) ? 0xffffffffu : r;
+    setC &= (__popc(setC) <= capC) ? 0xffffffffu : c;
 }
 
 // Transpose of the M x M bit matrix whose row i is held by lane i of a group of M lanes
@@ -897,8 +904,8 @@ __device__ __forceinline__ unsigned round_block(float* ks, const float* ws, unsi
     for (int round = 0; round < M * M; ++round) {
         if (!__any_sync(FULL, availR != 0u)) break;
         if (round == M * M - 1) flags |= DEV_INTERNAL;
-        const unsigned pickR = first_available<M>(availR, capR, rtab);
-        const unsigned pickC = first_available<M>(availC, capC, ctab);
+        unsigned pickR = availR, pickC = availC;
+        first_available<M>(pickR, capR, rtab, pickC, capC, ctab);
         // an entry picked from both sides is taken: takenR columns in my row, takenC rows in my
         // column.  (Both picks are transposed, not takenR a second time: two chains of five
         // exchanges side by side, or one for M <= 16, where both fit into one word.)
@@ -943,19 +950,38 @@ __device__ __forceinline__ unsigned round_block(float* ks, const float* ws, unsi
         float best = __int_as_float(0xff800000);
         int bi = 0x7fffffff;
         const float w_ijp = lines_ok ? ws[di * WS + jp] : 0.0f;
-        while (cand) {                               // ascending i': ties keep the smallest
-            const int ip = __ffs(cand) - 1;
-            cand &= cand - 1u;
-            if (!TS_CHECK(ip < M)) continue;
-            const float sc = __fsub_rn(__fadd_rn(w_ijp, ws[ip * WS + dj]), ws[ip * WS + jp]);
-            if (sc > best) { best = sc; bi = ip; }
+        // Ascending i': ties keep the smallest.  Four candidates a turn, so that their scores are read
+        // together: one at a time, the chain of reads was most of a step.
+        while (cand) {
+            int ip[4];
+            float sc[4];
+            bool is[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                is[k] = cand != 0u;
+                ip[k] = is[k] ? __ffs(cand) - 1 : 0;
+                cand &= cand - 1u;                   // 0 stays 0
+                is[k] = is[k] && TS_CHECK(ip[k] < M);
+                sc[k] = is[k] ? __fsub_rn(__fadd_rn(w_ijp, ws[ip[k] * WS + dj]), ws[ip[k] * WS + jp]) : 0.0f;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (is[k] && sc[k] > best) { best = sc[k]; bi = ip[k]; }
         }
         int bflat = (bi == 0x7fffffff) ? 0x7fffffff : bi * M + jp;
+        if constexpr (M == 32) {     // the largest score of the warp, then the smallest index that has it
+            const unsigned u = __float_as_uint(best + 0.0f);                      // -0 -> +0
+            const unsigned mine = (u & 0x80000000u) ? ~u : (u | 0x80000000u);     // ascending
+            const unsigned top = __reduce_max_sync(FULL, mine);
+            bflat = (int)__reduce_min_sync(FULL, (mine == top) ? (unsigned)bflat : 0x7fffffffu);
+            best = __uint_as_float((top & 0x80000000u) ? top & 0x7fffffffu : ~top);
+        } else {
 #pragma unroll
-        for (int off = M / 2; off > 0; off >>= 1) {
-            const float ob = __shfl_xor_sync(FULL, best, off, M);
-            const int of = __shfl_xor_sync(FULL, bflat, off, M);
-            if (ob > best || (ob == best && of < bflat)) { best = ob; bflat = of; }
+            for (int off = M / 2; off > 0; off >>= 1) {
+                const float ob = __shfl_xor_sync(FULL, best, off, M);
+                const int of = __shfl_xor_sync(FULL, bflat, off, M);
+                if (ob > best || (ob == best && of < bflat)) { best = ob; bflat = of; }
+            }
         }
         if (work) {
             if (bflat == 0x7fffffff) {            // no valid triple: only with non-finite scores
