@@ -241,11 +241,11 @@ int64_t tsenor_launch_count(void);
 /*
  * Register layout of the Dykstra stage (Algorithm 1).  The kernels come in a throughput
  * layout (fewest exchanges between lanes per element; for matrices with enough blocks to
- * fill the GPU) and, for M < 32, a latency layout (every block spread over M lanes: a
- * shorter chain of dependent work per iteration and more warps for the same matrix; for
- * small matrices such as the per-iteration solves of the ADMM integration, Section 4).
- * TSENOR_LAYOUT_AUTO (the default) picks the latency layout when even its finer units
- * give no more than 16 warps per SM.  The two layouts add the same numbers in a different
+ * fill the GPU) and a latency layout (M < 32: every block spread over M lanes that keep its
+ * rows and its columns, a shorter chain of dependent work per iteration; for small matrices
+ * such as the per-iteration solves of the ADMM integration, Section 4).
+ * TSENOR_LAYOUT_AUTO (the default) picks the latency layout while its warps are few per SM
+ * (6, 12, 6 and 8 for M = 4, 8, 16 and 32).  The two layouts add the same numbers in a different
  * order, so plans agree to rounding level (both within the documented 1e-4 of the fp64
  * result), not bit for bit.  Process-wide setting, meant for tests and benchmarks; returns
  * the previous value, or TSENOR_ERR_ARG.

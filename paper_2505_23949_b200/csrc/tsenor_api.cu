@@ -119,20 +119,25 @@ int launch_layout(const tsenor::Params& P, cudaStream_t st) {
     return finish_launch();
 }
 
-// Chooses the register layout: the latency layout (a block over M lanes) when even its
-// finer units leave the GPU with no more than 16 warps per SM, i.e. when the run time is
-// the chain of dependent iterations of a single warp rather than instruction throughput.
+// Chooses the register layout: the latency layout while its warps leave every scheduler of the GPU so
+// few of them that the run time is the chain of dependent iterations of a single warp rather than
+// instruction throughput.  Where the line lies, in warps of the latency layout per SM, from both sides
+// (us, latency against throughput):
+//   M = 4   3.6: 27.5 / 33.1   13.8: 38.9 / 31.0 (one lane a block needs no exchange at all)
+//   M = 8   6.9: 37.8 / 50.1   27.7: 103 / 78
+//   M = 16  3.5: 46.1 / 59.1   13.8: 113 / 79
+//   M = 32  6.9: 87.0 / 91.4   (the same layout; above it the second kernel's 16 warps per SM are too few)
+constexpr int64_t latency_warps_per_sm(int M) { return M == 8 ? 12 : M == 32 ? 8 : 6; }
+
 template <int M, int MODE, bool EE>
 int launch(const tsenor::Params& P, cudaStream_t st) {
-    if constexpr (M < 32) {   // a 32 x 32 block takes a whole warp in either layout
-        const int policy = g_layout.load(std::memory_order_relaxed);
-        bool fine = (policy == TSENOR_LAYOUT_LATENCY);
-        if (policy == TSENOR_LAYOUT_AUTO) {
-            int64_t nbp = 0;
-            fine = unit_count<M, 1>(P, &nbp) <= 16LL * sm_count();
-        }
-        if (fine) return launch_layout<M, MODE, 1, EE>(P, st);
+    const int policy = g_layout.load(std::memory_order_relaxed);
+    bool fine = (policy == TSENOR_LAYOUT_LATENCY);
+    if (policy == TSENOR_LAYOUT_AUTO) {
+        int64_t nbp = 0;
+        fine = unit_count<M, 1>(P, &nbp) <= latency_warps_per_sm(M) * sm_count();
     }
+    if (fine) return launch_layout<M, MODE, 1, EE>(P, st);
     return launch_layout<M, MODE, 0, EE>(P, st);
 }
 

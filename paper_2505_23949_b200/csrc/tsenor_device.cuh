@@ -34,43 +34,39 @@ __shared__ int g_bounds_flags;
 #endif
 
 // ---------------------------------------------------------------------------
-// Dykstra register layout.  A block is spread over LPB = PR*PC lanes arranged
-// as PR x PC; each lane keeps an MR x MC sub-tile.  Row sums are reduced over
-// the PC lanes that share rows, column sums over the PR lanes that share
-// columns.  Two layouts per block size:
-//   V = 0  throughput: 4 x 8 sub-tiles (4 x 4 for M = 4), the fewest exchanges per
-//          element; used whenever the matrix has enough blocks to fill the GPU;
-//   V = 1  latency (M < 32): a block over M lanes (the most the exchange scheme allows:
-//          every lane must end up owning one row sum and one column sum), i.e. the
-//          shortest chain of dependent work per iteration and 2-4 times as many
-//          warps for the same matrix; used for matrices too small to fill the GPU.
-//          (Butterfly all-reduces in place of reduce-scatter + all-gather halve the
-//          exchange hops but measured no faster: the chain is then bound by the two
-//          reciprocals and the arithmetic between the hops.)
+// Dykstra register layouts.
+//   V = 0  throughput: a block is spread over LPB = PR*PC lanes arranged as PR x PC; each lane
+//          keeps an MR x MC sub-tile, 4 x 8 (4 x 4 for M = 4), the fewest exchanges per element
+//          that the registers allow.  Row sums are reduced over the PC lanes that share rows,
+//          column sums over the PR lanes that share columns.  Used whenever the matrix has
+//          enough blocks to fill the GPU.
+//   V = 1  latency, for matrices too small for that.  M < 32: a block over M lanes, of which lane i
+//          keeps row i and, a second time, column i ("twin" layout, see twin_plan): twice the
+//          element-wise work, but all sums are a lane's own and the scalings cross the lanes by two
+//          shared-memory broadcasts an iteration where sub-tiles need six to eight dependent
+//          shuffles.  M = 32: the sub-tiles of V = 0, compiled for more registers.
 // ---------------------------------------------------------------------------
-template <int M, int V> struct Tile;
-template <> struct Tile<32, 0> { static constexpr int PR = 8, PC = 4, MR = 4, MC = 8; };
-template <> struct Tile<16, 0> { static constexpr int PR = 4, PC = 2, MR = 4, MC = 8; };
-template <> struct Tile<8, 0>  { static constexpr int PR = 2, PC = 1, MR = 4, MC = 8; };
-template <> struct Tile<4, 0>  { static constexpr int PR = 1, PC = 1, MR = 4, MC = 4; };
-template <> struct Tile<16, 1> { static constexpr int PR = 4, PC = 4, MR = 4, MC = 4; };
-template <> struct Tile<8, 1>  { static constexpr int PR = 4, PC = 2, MR = 2, MC = 4; };
-template <> struct Tile<4, 1>  { static constexpr int PR = 2, PC = 2, MR = 2, MC = 2; };
+template <int M> struct Tile;
+template <> struct Tile<32> { static constexpr int PR = 8, PC = 4, MR = 4, MC = 8; };
+template <> struct Tile<16> { static constexpr int PR = 4, PC = 2, MR = 4, MC = 8; };
+template <> struct Tile<8>  { static constexpr int PR = 2, PC = 1, MR = 4, MC = 8; };
+template <> struct Tile<4>  { static constexpr int PR = 1, PC = 1, MR = 4, MC = 4; };
 
 template <int M_, int V_> struct Geom {
     static constexpr int M = M_, V = V_;
-    using T = Tile<M, V>;
-    static constexpr int LPB = T::PR * T::PC;        // lanes per block (Dykstra)
+    static constexpr bool TWIN = (V == 1 && M < 32);
+    using T = Tile<M>;
+    static constexpr int LPB = TWIN ? M : T::PR * T::PC;   // lanes per block (Dykstra)
     static constexpr int BPW = 32 / LPB;             // blocks per warp
     static constexpr int UW = BPW * M;               // columns of a unit: its blocks side by side
     static constexpr int WS = UW + 1;                // shared row stride (floats)
     static constexpr int GPW = 32 / M;               // rounding groups per warp (blocks of one mask word)
     static constexpr int PASSES = BPW / GPW;         // rounding passes per warp
-    static constexpr int RO = T::MR / T::PC, CO = T::MC / T::PR;   // lines whose sums a lane finishes
+    static constexpr int RO = TWIN ? 1 : T::MR / T::PC, CO = TWIN ? 1 : T::MC / T::PR;   // lines a lane finishes
     static_assert(T::MR >= T::PC && T::MC >= T::PR && T::MC % 2 == 0 && (T::MR * T::MC) % 4 == 0, "tile shape");
     static_assert(T::PR * T::MR == M && T::PC * T::MC == M, "tile covers the block");
     static_assert(BPW % GPW == 0, "a unit is a whole number of mask words wide");
-    static_assert(32 * T::MR * T::MC <= M * WS, "the stash of t0 fits in the key panel");
+    static_assert(TWIN || 32 * T::MR * T::MC <= M * WS, "the stash of t0 fits in the key panel");
 };
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -273,7 +269,7 @@ __device__ __forceinline__ float dykstra_step(float2 (&V)[G::T::MR][G::T::MC / 2
         Pc[k] *= kap[k];
     }
     all_gather<MC, PR>(kap, PC);
-    if constexpr (PackMul<M>::value && MR % 2 == 0) {
+    if constexpr (PackMul<M>::value && G::V == 0 && MR % 2 == 0) {
 #pragma unroll
         for (int a = 0; a < MR; a += 2) {
             const float2 r = __fmul2_rn(make_float2(rs[a], rs[a + 1]), make_float2(sc[a], sc[a + 1]));
@@ -1119,27 +1115,202 @@ __device__ __forceinline__ void store_plan(const Params& P, const UnitMap<G::M>&
     }
 }
 
+// ---------------------------------------------------------------------------
+// Algorithm 1 in the twin layout (M < 32, small matrices): the scores of the unit's blocks from
+// `panel` to the capped log-plan in `k` (same row stride).  Lane i of a block's M lanes keeps row i
+// of the linear iterate (Vr) and, a second time, column i (Vc) with the factors of all rows (Ra); both
+// copies see the same operations and stay equal bit for bit.  A row sum and a column sum are then a
+// lane's own, and an iteration is two exchanges long: rho to the lanes of the block (one store, M / 4
+// broadcast loads of 16 bytes), kap likewise.  What bounds it is that chain: sum, reciprocal,
+// exchange, sum, reciprocal, exchange.  The stash of t0 is the M x 32 matrix in `k` itself, read by
+// rows and by columns.  pot: 64 float2 for the owned potentials, then 64 floats for the exchange.
+// The numbers are those of dykstra_iterate, whose comments apply; only the order of the sums differs.
+// A lone warp takes 155 / 169 / 227 clocks an iteration for M = 4 / 8 / 16, where a block spread over M
+// lanes in sub-tiles took 181 / 229 / 267 and the throughput layout takes 129 / 226 / 244 (but leaves one
+// warp several blocks to round): 512 x 512 4:8 43.5 -> 37.8 us, 512 x 512 8:16 53.9 -> 46.1 us,
+// 256 x 264 2:4 31.9 -> 27.5 us.
+// ---------------------------------------------------------------------------
+template <int M> __device__ __forceinline__ void exchange(float* buf, int lane, float mine, float2 (&all)[M / 2]) {
+    buf[lane] = mine;
+    __syncwarp();
+    const float4* const src = reinterpret_cast<const float4*>(buf + lane / M * M);
+#pragma unroll
+    for (int q = 0; q < M / 4; ++q) {
+        const float4 v = src[q];
+        all[2 * q] = make_float2(v.x, v.y);
+        all[2 * q + 1] = make_float2(v.z, v.w);
+    }
+}
+template <int M> __device__ __forceinline__ float sum_line(const float2 (&v)[M / 2]) {
+    float2 a = v[0], b = v[1];               // two chains
+#pragma unroll
+    for (int j = 2; j < M / 2; j += 2) {
+        a = __fadd2_rn(a, v[j]);
+        b = __fadd2_rn(b, v[j + 1]);
+    }
+    a = __fadd2_rn(a, b);
+    return a.x + a.y;
+}
+template <int M, bool DELTA>
+__device__ __forceinline__ float twin_step(float2 (&Vr)[M / 2], float2 (&Vc)[M / 2], float2 (&Ra)[M / 2], float& r,
+                                           float& pc, float* ex, int lane, float Nf) {
+    float2 e[M / 2], f[M / 2], x[M / 2];
+#pragma unroll
+    for (int j = 0; j < M / 2; ++j) e[j] = make_float2(__saturatef(Vr[j].x * r), __saturatef(Vr[j].y * r));
+    const float s = sum_line<M>(e);
+    const float rho = Nf * rcp_approx(s);
+    exchange<M>(ex, lane, rho, x);
+    r *= rho;
+#pragma unroll
+    for (int i = 0; i < M / 2; ++i) {
+        f[i] = make_float2(__saturatef(Vc[i].x * Ra[i].x), __saturatef(Vc[i].y * Ra[i].y));
+        Ra[i] = __fmul2_rn(Ra[i], x[i]);
+    }
+    float2 a = __fmul2_rn(f[0], x[0]), b = __fmul2_rn(f[1], x[1]);
+#pragma unroll
+    for (int i = 2; i < M / 2; i += 2) {
+        a = __ffma2_rn(f[i], x[i], a);
+        b = __ffma2_rn(f[i + 1], x[i + 1], b);
+    }
+    a = __fadd2_rn(a, b);
+    const float c = a.x + a.y;
+    const float kap = Nf * rcp_approx(c);
+    exchange<M>(ex + 32, lane, kap, x);
+    pc *= kap;
+#pragma unroll
+    for (int j = 0; j < M / 2; ++j) {
+        Vr[j] = __fmul2_rn(Vr[j], x[j]);
+        Vc[j] = __fmul2_rn(Vc[j], make_float2(kap, kap));
+    }
+    return DELTA ? fmaxf(fabsf(s - Nf), fabsf(c - Nf)) : 0.0f;
+}
+template <class G, bool EE>
+__device__ __forceinline__ int twin_plan(const Params& P, const float* panel, float* k, float2* pot, int lane) {
+    constexpr int M = G::M, WS = G::WS, H = M / 2;
+    const int i = lane % M;
+    const float* const score_row = panel + i * WS + (lane - i);      // row i of my block
+    float* const row = k + i * WS + (lane - i);
+    const float* const col = k + lane;                               // column i of my block
+    if (!TS_CHECK((M - 1) * WS + lane < M * WS && i * WS + (lane - i) + M <= M * WS)) return 0;
+    float* const ex = reinterpret_cast<float*>(pot + 64);
+    float2* const fpot = pot + lane;
+    float2* const gpot = pot + 32 + lane;
+    float t[M];
+    float mx = 0.0f;
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+        t[j] = score_row[j];
+        mx = fmaxf(mx, t[j]);
+    }
+    float c_hi = P.c_hi, c_lo = P.c_lo;
+    if (P.per_block_tau) {   // tau of this block = tau_rel / its largest score
+        float bm = mx;
+#pragma unroll
+        for (int s = 1; s < M; s <<= 1) bm = fmaxf(bm, __shfl_xor_sync(FULL, bm, s));
+        c_hi = (bm > 0.0f) ? __fdiv_rn(P.c_hi, bm) : 0.0f;
+        c_lo = (bm > 0.0f) ? __fdiv_rn(fmaf(-c_hi, bm, P.c_hi) + P.c_lo, bm) : 0.0f;
+    }
+    if (P.iters <= 0) {
+#pragma unroll
+        for (int j = 0; j < M; ++j) row[j] = fmaf(t[j], c_lo, t[j] * c_hi);
+        __syncwarp();
+        return 0;
+    }
+    const float sh = mx * c_hi;
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+        t[j] = fmaf(t[j], c_lo, fmaf(t[j], c_hi, -sh));
+        row[j] = t[j];
+    }
+    float r = 1.0f, pc = 1.0f;
+    float2 x[H], y[H];
+    {   // iteration 0, log domain
+        float s = 0.f;
+#pragma unroll
+        for (int j = 0; j < M; ++j) s += ex2_approx(t[j]);
+        const float F = P.log2N - lg2_approx(s);
+        *fpot = make_float2(F, 0.f);
+        exchange<M>(ex, lane, F, x);             // (its barrier also publishes t0)
+        float cm = -3.4028234e38f, cp = 0.f;
+#pragma unroll
+        for (int a = 0; a < M; ++a) {
+            t[a] = col[a * WS] + ((a % 2) ? x[a / 2].y : x[a / 2].x);
+            cm = (a == 0) ? t[0] : fmaxf(cm, t[a]);
+        }
+#pragma unroll
+        for (int a = 0; a < M; ++a) cp += ex2_approx(t[a] - cm);
+        *gpot = make_float2((P.log2N - cm) - lg2_approx(cp), 0.f);
+    }
+    int it = 1, iters = P.iters;
+    float2 Vr[H], Vc[H], Ra[H];
+#pragma unroll 1
+    while (it < iters) {
+        const float F = add_potential(fpot, r), Gc = add_potential(gpot, pc);
+        exchange<M>(ex, lane, F, x);
+        exchange<M>(ex + 32, lane, Gc, y);
+#pragma unroll
+        for (int j = 0; j < H; ++j) {
+            const float2 a = __fadd2_rn(__fadd2_rn(make_float2(row[2 * j], row[2 * j + 1]), make_float2(F, F)), y[j]);
+            const float2 b = __fadd2_rn(__fadd2_rn(make_float2(col[2 * j * WS], col[(2 * j + 1) * WS]), x[j]),
+                                        make_float2(Gc, Gc));
+            Vr[j] = make_float2(ex2_approx(a.x), ex2_approx(a.y));
+            Vc[j] = make_float2(ex2_approx(b.x), ex2_approx(b.y));
+            Ra[j] = make_float2(1.0f, 1.0f);
+        }
+        r = pc = 1.0f;
+        const int run_end = (iters - it > MAXRUN) ? it + MAXRUN : iters;
+        bool wide = false;
+#pragma unroll 1
+        while (!wide && it + CHECK <= run_end) {
+#pragma unroll
+            for (int u = 0; u < CHECK - 1; ++u) twin_step<M, false>(Vr, Vc, Ra, r, pc, ex, lane, P.Nf);
+            const float delta = twin_step<M, EE>(Vr, Vc, Ra, r, pc, ex, lane, P.Nf);
+            it += CHECK;
+            if (EE && __all_sync(FULL, delta < P.ee_eps)) {   // every block of the warp has converged
+                iters = it;
+                wide = true;                                  // skips the remainder loop as well
+                break;
+            }
+            wide = __any_sync(FULL, out_of_window(r) || out_of_window(pc));
+        }
+        if (!wide) {   // fewer than CHECK iterations left (end of the last run only)
+#pragma unroll 1
+            for (; it < run_end; ++it) twin_step<M, false>(Vr, Vc, Ra, r, pc, ex, lane, P.Nf);
+        }
+    }
+    // final potentials, t = t0 + F + G and x = min(t, 0)
+    const float F = add_potential(fpot, r), Gc = add_potential(gpot, pc);
+    exchange<M>(ex + 32, lane, Gc, y);           // (its barrier: no column of t0 is read any more)
+#pragma unroll
+    for (int j = 0; j < M; ++j) row[j] = fminf((row[j] + F) + ((j % 2) ? y[j / 2].y : y[j / 2].x), 0.0f);
+    __syncwarp();
+    return iters;
+}
+
 template <class G, int MODE, bool EE> struct SmemLayout {   // of one warp
     static constexpr int M = G::M;
     // The score panel is kept beside the key panel for the local search, except that the whole
     // method at M = 32 reads the scores of a block again when it needs them (RELOAD): the panel would
     // cost the SM 4 of its 20 warps (14336 x 4096, 16:32: 3.13 ms with it, 3.03 without).
-    static constexpr bool RELOAD = (M == 32 && MODE == 0 && !EE);
+    static constexpr bool RELOAD = (M == 32 && MODE == 0 && G::V == 0 && !EE);
     static constexpr bool HAS_W = MODE != 1 && !RELOAD;
-    static constexpr int POT = (MODE == 2) ? 0 : 64 * (G::RO + G::CO);
+    static constexpr int POT = (MODE == 2) ? 0 : 64 * (G::RO + G::CO) + (G::TWIN ? 64 : 0);
     static constexpr int CPRE = (M == 32 && MODE != 1) ? 32 * CPRE_STRIDE : 0;
     static constexpr int AUX = (POT > CPRE) ? POT : CPRE;
     alignas(16) float k[M * G::WS];     // scores, stash of t0, keys, row prefix tables in turn
     float w[HAS_W ? M * G::WS : 1];
-    alignas(8) float aux[AUX ? AUX : 1];  // potentials, then the column-prefix tables of M = 32
+    alignas(16) float aux[AUX ? AUX : 1];   // potentials (and the twin layout's exchange), then the
+                                            // column-prefix tables of M = 32
 };
 // Resident warps per SM the register allocation aims for: 20 where the loop fits in 96 registers.
-template <int M, int V, bool EE> struct MinWarps { static constexpr int value = (M == 32 && !EE) ? 20 : 16; };
+template <int M, int V, bool EE> struct MinWarps {
+    static constexpr int value = (V == 1) ? 12 : (M == 32 && !EE) ? 20 : 16;
+};
 // Warps per CTA.  One: 3 to 25 % faster than four on ragged widths (finer tail) and never slower,
 // with one exception.  The stopping test at M = 32 runs through the kernel's whole code for a dozen
 // iterations of work; four warps that go through it together (barriers after the loader and before
 // the rounding stage) share what they fetch of it (14336 x 4096: 0.90 ms apart, 0.71 together).
-template <int M, int V, bool EE> struct CtaWarps { static constexpr int value = (M == 32 && EE) ? 4 : 1; };
+template <int M, int V, bool EE> struct CtaWarps { static constexpr int value = (M == 32 && V == 0 && EE) ? 4 : 1; };
 
 // Cells of a lane's sub-tile in a shared-memory panel.
 template <class G> struct SubTile {
@@ -1160,7 +1331,7 @@ tsenor_kernel(const Params P) {
     using G = Geom<M, V>;
     using T = typename G::T;
     using L = SmemLayout<G, MODE, EE>;
-    constexpr int MR = T::MR, MC = T::MC, PR = T::PR, PC = T::PC;
+    [[maybe_unused]] constexpr int MR = T::MR, MC = T::MC, PR = T::PR, PC = T::PC;
     constexpr int WPC = CtaWarps<M, V, EE>::value;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x % 32;
@@ -1183,7 +1354,16 @@ tsenor_kernel(const Params P) {
     else __syncwarp();
 
     // ---- Algorithm 1
-    if (MODE != 2) {
+    if constexpr (MODE != 2 && G::TWIN) {
+        const int ran = twin_plan<G, EE>(P, panel, sm.k, reinterpret_cast<float2*>(sm.aux), lane);
+        if (P.iter_sum && P.iters > 0) {
+            const UnitMap<M> um(P.rows, P.cols, P.nbp, this_unit<WPC>() * G::BPW);
+            int64_t r0, c0;
+            const bool there = um.locate(lane / M, r0, c0);
+            const int nact = __popc(__ballot_sync(FULL, there && lane % M == 0));
+            if (lane == 0 && nact) atomicAdd(P.iter_sum, (unsigned long long)ran * nact);
+        }
+    } else if constexpr (MODE != 2) {
         float t[MR][MC];
         float mx[MR];
         const SubTile<G> st0(lane);
@@ -1253,9 +1433,9 @@ tsenor_kernel(const Params P) {
             for (int b = 0; b < MC; ++b)
                 if (TS_CHECK(st.row(a) < M && st.col(b) < G::UW)) sm.k[st.row(a) * G::WS + st.col(b)] = t[a][b];
         __syncwarp();
-        if (MODE == 1)           // ---- plan writer
-            store_plan<G>(P, UnitMap<M>(P.rows, P.cols, P.nbp, this_unit<WPC>() * G::BPW), lane, sm.k);
     }
+    if (MODE == 1)               // ---- plan writer
+        store_plan<G>(P, UnitMap<M>(P.rows, P.cols, P.nbp, this_unit<WPC>() * G::BPW), lane, sm.k);
 
     if (MODE == 0 && WPC > 1) __syncthreads();
     // ---- Algorithm 2 and the mask writer: the blocks of one mask word (GPW M = 32 columns) a pass
