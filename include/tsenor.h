@@ -245,7 +245,7 @@ int64_t tsenor_launch_count(void);
  * rows and its columns, a shorter chain of dependent work per iteration; for small matrices
  * such as the per-iteration solves of the ADMM integration, Section 4).
  * TSENOR_LAYOUT_AUTO (the default) picks the latency layout while its warps are few per SM
- * (6, 12, 6 and 8 for M = 4, 8, 16 and 32).  The two layouts add the same numbers in a different
+ * (6, 12, 6 and 16 for M = 4, 8, 16 and 32).  The two layouts add the same numbers in a different
  * order, so plans agree to rounding level (both within the documented 1e-4 of the fp64
  * result), not bit for bit.  Process-wide setting, meant for tests and benchmarks; returns
  * the previous value, or TSENOR_ERR_ARG.

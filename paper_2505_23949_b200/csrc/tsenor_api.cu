@@ -126,8 +126,13 @@ int launch_layout(const tsenor::Params& P, cudaStream_t st) {
 //   M = 4   3.6: 27.5 / 33.1   13.8: 38.9 / 31.0 (one lane a block needs no exchange at all)
 //   M = 8   6.9: 37.8 / 50.1   27.7: 103 / 78
 //   M = 16  3.5: 46.1 / 59.1   13.8: 113 / 79
-//   M = 32  6.9: 87.0 / 91.4   (the same layout; above it the second kernel's 16 warps per SM are too few)
-constexpr int64_t latency_warps_per_sm(int M) { return M == 8 ? 12 : M == 32 ? 8 : 6; }
+//   M = 32  6.9: 85.1 / 92.0   15.6: 142.4 / 145.7 (the same layout, as long as all its warps are resident)
+constexpr int64_t latency_warps_per_sm(int M) { return M == 8 ? 12 : M == 32 ? 16 : 6; }
+// Rounding alone has no iterations to share lanes for, and the latency layout's units are one rounding
+// pass: more warps and nothing serial (2048 x 2048, us against the wider units: M = 8 20.8 / 24.4, M = 16
+// 22.5 / 27.2; 4096 x 4096 86.7 / 85.8 and 88.5 / 100.4).  At M = 4 a pass is so short that the wider units
+// win once the GPU is full (2048 x 2048 23.6 / 21.7; the line is at 1024 x 1024).
+constexpr int64_t rounding_warps_per_sm(int M) { return M == 4 ? 64 : M == 32 ? 0 : INT64_MAX >> 16; }
 
 template <int M, int MODE, bool EE>
 int launch(const tsenor::Params& P, cudaStream_t st) {
@@ -135,9 +140,18 @@ int launch(const tsenor::Params& P, cudaStream_t st) {
     bool fine = (policy == TSENOR_LAYOUT_LATENCY);
     if (policy == TSENOR_LAYOUT_AUTO) {
         int64_t nbp = 0;
-        fine = unit_count<M, 1>(P, &nbp) <= latency_warps_per_sm(M) * sm_count();
+        const int64_t line = (MODE == 2) ? rounding_warps_per_sm(M) : latency_warps_per_sm(M);
+        fine = unit_count<M, 1>(P, &nbp) <= line * sm_count();
     }
     if (fine) return launch_layout<M, MODE, 1, EE>(P, st);
+    if constexpr (M == 16 && MODE != 2 && !EE) {
+        // In between, a few warps to a scheduler: the build of the throughput layout with the shorter
+        // chain (16 warps per SM, nothing extra packed) as long as all of them are resident at once
+        // (1024 x 1024, 6.9 warps per SM: 78.8 us against 87.0; 4096 x 4096, 111: 870 against 857).
+        int64_t nbp = 0;
+        if (policy == TSENOR_LAYOUT_AUTO && unit_count<M, 2>(P, &nbp) <= 16LL * sm_count())
+            return launch_layout<M, MODE, 2, EE>(P, st);
+    }
     return launch_layout<M, MODE, 0, EE>(P, st);
 }
 

@@ -45,6 +45,7 @@ __shared__ int g_bounds_flags;
 //          element-wise work, but all sums are a lane's own and the scalings cross the lanes by two
 //          shared-memory broadcasts an iteration where sub-tiles need six to eight dependent
 //          shuffles.  M = 32: the sub-tiles of V = 0, compiled for more registers.
+//   V = 2  M = 16 in between: the sub-tiles of V = 0, compiled for the shorter chain.
 // ---------------------------------------------------------------------------
 template <int M> struct Tile;
 template <> struct Tile<32> { static constexpr int PR = 8, PC = 4, MR = 4, MC = 8; };
@@ -197,10 +198,17 @@ __device__ __forceinline__ float add_potential(float2* p, float prod) {
 constexpr int CHECK = 4;     // iterations between range tests of the accumulated scalings
 constexpr int MAXRUN = 48;   // longest run of linear-domain iterations (multiple of CHECK)
 
+// Exponent field outside [127-16, 127+16] <=> product outside [2^-16, 2^17).  A product that is inf or
+// NaN (exponent field 255: a block poisoned by a non-finite score) does not vote, so that it cannot
+// change when the other blocks of its warp rebuild.
 __device__ __forceinline__ bool out_of_window(float p) {
     const unsigned e = (__float_as_uint(p) >> 23) & 0xffu;
     return (e - 111u) > 32u && e != 255u;
 }
+
+// Products in the window, and no others, are at most WINDOW from its lower end as bit patterns.
+constexpr unsigned WINDOW = (33u << 23) - 1u;
+__device__ __forceinline__ unsigned window_distance(float p) { return __float_as_uint(p) - (111u << 23); }
 
 // One iteration t >= 1 on the linear-domain iterate.  Element-wise work runs on
 // pairs of columns with the packed fp32x2 add / mul / fma of sm_100 (half the
@@ -211,24 +219,28 @@ __device__ __forceinline__ bool out_of_window(float p) {
 // give rho_i = N / sum, column sums are sum_i e_ij rho_i, R_i <- R_i rho_i in every
 // lane of the row.  (The other form, min(V, 1/R_i) with the clip threshold moving
 // instead of the tile, needs the half-rate ALU pipe for the min and a second gather
-// for the thresholds: slower at every size, by 3 % for M = 4 and M = 8.)
+// for the thresholds: slower at every size, by 3 % for M = 8 and 6 % for M = 4.  The clip's
+// product is one more rounding than the min has: at N = 1, M = 4 the log-plan is 1.1 to 1.4 times as
+// far from the fp64 iterate, 2e-7 relative; at the other sizes and for the plan itself there is no
+// difference on average.)
 //
-// Whether the exchanges' adds and the row factors are packed too is a matter of how the
-// packed and the scalar instructions of the other warps interleave on the FMA pipes, and
-// was measured for each size (1 to 2 %).
-template <int M> struct PackAdd { static constexpr bool value = (M == 8); };
-template <int M> struct PackMul { static constexpr bool value = (M == 8 || M == 32); };
+// Whether the exchanges' adds and the row factors are packed too (PACK) is a matter of how the
+// packed and the scalar instructions of the other warps interleave on the FMA pipes: the factors
+// gain 1 to 2 % at every size, the adds as much for M >= 16 and nothing for M = 8.  A lone warp, and
+// the stopping test's mixture, only see the packed ones' longer latency (14336 x 32: 69.4 us
+// without, 74.5 with).
+template <int M> struct PackAdd { static constexpr bool value = (M >= 16); };
 
 // DELTA: also returns this lane's share of the marginal violation seen by the iteration,
 // max over the lines it owns of |row sum of e - N| and |column sum of e rho - N|.
-template <class G, bool DELTA = false>
+template <class G, bool PACK, bool DELTA = false>
 __device__ __forceinline__ float dykstra_step(float2 (&V)[G::T::MR][G::T::MC / 2], float (&rs)[G::T::MR],
                                               float (&Pc)[G::CO], float Nf) {
     using T = typename G::T;
     constexpr int M = G::M;
     constexpr int MR = T::MR, MC = T::MC, PR = T::PR, PC = T::PC;
     constexpr int RO = G::RO, CO = G::CO, MP = MC / 2;
-    using Add = typename std::conditional<PackAdd<M>::value, OpAdd2, OpAdd>::type;
+    using Add = typename std::conditional<PACK && PackAdd<M>::value, OpAdd2, OpAdd>::type;
     float2 m[MR][MP];
     float rp[MR], sc[MR], cp[MC], kap[MC];
 #pragma unroll
@@ -269,7 +281,7 @@ __device__ __forceinline__ float dykstra_step(float2 (&V)[G::T::MR][G::T::MC / 2
         Pc[k] *= kap[k];
     }
     all_gather<MC, PR>(kap, PC);
-    if constexpr (PackMul<M>::value && G::V == 0 && MR % 2 == 0) {
+    if constexpr (PACK) {
 #pragma unroll
         for (int a = 0; a < MR; a += 2) {
             const float2 r = __fmul2_rn(make_float2(rs[a], rs[a + 1]), make_float2(sc[a], sc[a + 1]));
@@ -297,6 +309,7 @@ __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], f
     constexpr int MR = T::MR, MC = T::MC, PR = T::PR, PC = T::PC;
     constexpr int RO = G::RO, CO = G::CO;
     constexpr int MP = MC / 2, NQ = MR * MC / 4;
+    constexpr bool PACK = (G::V == 0 && !EE);
     float F[MR], Gc[MC];
     float rs[MR];
     float Pc[CO];              // products of kap since the last rebuild; those of rho are rs[0 .. RO)
@@ -382,9 +395,9 @@ __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], f
 #pragma unroll 1
         while (!wide && it + CHECK <= run_end) {
 #pragma unroll(EE && G::M == 32 ? 1 : CHECK)   // (the stopping test at M = 32 is mostly code that runs once)
-            for (int u = 0; u < CHECK - 1; ++u) dykstra_step<G>(V, rs, Pc, Nf);
+            for (int u = 0; u < CHECK - 1; ++u) dykstra_step<G, PACK>(V, rs, Pc, Nf);
             if constexpr (EE) {
-                const float delta = dykstra_step<G, true>(V, rs, Pc, Nf);
+                const float delta = dykstra_step<G, PACK, true>(V, rs, Pc, Nf);
                 if (__all_sync(FULL, delta < ee_eps)) {   // every block of the warp has converged
                     it += CHECK;
                     iters = it;
@@ -392,22 +405,29 @@ __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], f
                     break;
                 }
             } else {
-                dykstra_step<G>(V, rs, Pc, Nf);
+                dykstra_step<G, PACK>(V, rs, Pc, Nf);
             }
             it += CHECK;
-            // exponent field in [127-16, 127+16] <=> product in [2^-16, 2^17).  A product that
-            // is inf or NaN (exponent field 255: a block poisoned by a non-finite score) does
-            // not vote, so that it cannot change when the other blocks of its warp rebuild.
-            bool w = false;
+            // V = 0: a first, cheap test (a subtraction and a maximum per line, every four iterations)
+            // that also catches inf, NaN and zero; what it catches is looked at properly (1.5 to 4 %
+            // of the loop).  A lone warp waits longer for the second vote than it saves.
+            unsigned far = 0u;
 #pragma unroll
-            for (int k = 0; k < RO; ++k) w |= out_of_window(rs[k]);
+            for (int k = 0; k < RO; ++k) far = max(far, window_distance(rs[k]));
 #pragma unroll
-            for (int k = 0; k < CO; ++k) w |= out_of_window(Pc[k]);
-            wide = __any_sync(FULL, w);
+            for (int k = 0; k < CO; ++k) far = max(far, window_distance(Pc[k]));
+            if (G::V != 0 || __any_sync(FULL, far > WINDOW)) {
+                bool w = false;
+#pragma unroll
+                for (int k = 0; k < RO; ++k) w |= out_of_window(rs[k]);
+#pragma unroll
+                for (int k = 0; k < CO; ++k) w |= out_of_window(Pc[k]);
+                wide = __any_sync(FULL, w);
+            }
         }
         if (!wide) {   // fewer than CHECK iterations left (end of the last run only)
 #pragma unroll 1
-            for (; it < run_end; ++it) dykstra_step<G>(V, rs, Pc, Nf);
+            for (; it < run_end; ++it) dykstra_step<G, PACK>(V, rs, Pc, Nf);
         }
     }
     // final potentials and t = t0 + F + G
@@ -1304,7 +1324,7 @@ template <class G, int MODE, bool EE> struct SmemLayout {   // of one warp
 };
 // Resident warps per SM the register allocation aims for: 20 where the loop fits in 96 registers.
 template <int M, int V, bool EE> struct MinWarps {
-    static constexpr int value = (V == 1) ? 12 : (M == 32 && !EE) ? 20 : 16;
+    static constexpr int value = (V == 1) ? 12 : (M >= 16 && V == 0 && !EE) ? 20 : 16;
 };
 // Warps per CTA.  One: 3 to 25 % faster than four on ragged widths (finer tail) and never slower,
 // with one exception.  The stopping test at M = 32 runs through the kernel's whole code for a dozen
