@@ -194,30 +194,64 @@ __global__ void fill_mask_kernel(uint32_t* bits, int64_t rows, int64_t wpr, int6
 }
 
 // Walk over the quads (4 columns) of a matrix: quad idx is (row(idx), 4 * (idx - row(idx) * qpr)).
-// Rows by a multiplication with ceil(2^64 / qpr), exact while the quads number less than 2^32 (the
-// error of the quotient is then below idx / 2^64 < 1 / qpr); instead of a 64-bit division, some 100 instructions.
+// Rows by a 32-bit multiplication with magic = ceil(2^(31+L) / qpr), L = ceil(log2 qpr), exact while the
+// quads number less than 2^31: the quotient is then too large by less than idx / 2^31 / qpr < 1 / qpr.
 struct QuadWalk {
     int64_t qpr, nq;
-    unsigned long long magic;     // 0: divide
+    unsigned magic, shift;        // magic 0: divide
     __device__ __forceinline__ int64_t row(int64_t idx) const {
-        return magic ? (int64_t)__umul64hi((unsigned long long)idx, magic) : idx / qpr;
+        return magic ? (int64_t)(__umulhi((unsigned)idx, magic) >> shift) : idx / qpr;
     }
 };
 QuadWalk quad_walk(int64_t rows, int64_t cols) {
-    QuadWalk q;
+    QuadWalk q{};
     q.qpr = cols / 4;
     q.nq = rows * q.qpr;
-    q.magic = (q.qpr > 1 && q.nq < (1LL << 32)) ? ~0ULL / (unsigned long long)q.qpr + 1 : 0;
+    if (q.qpr > 1 && q.nq < (1LL << 31)) {
+        int L = 1;
+        while ((1LL << L) < q.qpr) ++L;
+        q.magic = (unsigned)(((1ULL << (31 + L)) + q.qpr - 1) / q.qpr);
+        q.shift = L - 1;
+    }
     return q;
+}
+
+// Aligned fp32 |W|, the common source of the scans: its quads are read four to a thread at once.  (The
+// other sources go through load_score_quad, whose branches keep a loop's reads from being batched.)
+constexpr int SCAN_U = 4;
+__device__ __forceinline__ bool plain_source(const tsenor::ScoreSrc& S) {
+    return S.kind == tsenor::SC_ABS && S.vec_w && !S.w_is_bf16;
+}
+__device__ __forceinline__ float4 load_plain_quad(const tsenor::ScoreSrc& S, int64_t r, int64_t c) {
+    return __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(S.w) + r * S.ld + c));
 }
 
 // Retained score of up to two masks under one score source (quads of 4 columns).
 __global__ void objective_kernel(const tsenor::ScoreSrc S, const uint32_t* __restrict__ bits_a,
                                  const uint32_t* __restrict__ bits_b, const QuadWalk q, int64_t wpr, double* out) {
     double acc_a = 0.0, acc_b = 0.0;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < q.nq;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        // (the division overlaps the fp64 adds here: 12 us for a 2048 x 2048 matrix with it, 13.5 with q.row)
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (!bits_b && plain_source(S)) {   // 14336 x 4096: 88 us a quad at a time, 50 this way
+        for (; idx + (SCAN_U - 1) * step < q.nq; idx += SCAN_U * step) {
+            float4 v[SCAN_U];
+            uint32_t m[SCAN_U];
+#pragma unroll
+            for (int u = 0; u < SCAN_U; ++u) {
+                const int64_t r = q.row(idx + u * step), c = (idx + u * step - r * q.qpr) * 4;
+                m[u] = bits_a[r * wpr + c / 32] >> (c % 32);
+                v[u] = load_plain_quad(S, r, c);
+            }
+#pragma unroll
+            for (int u = 0; u < SCAN_U; ++u) {
+                const float e[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if ((m[u] >> k) & 1u) acc_a += (double)fabsf(e[k]);
+            }
+        }
+    }
+    for (; idx < q.nq; idx += step) {
         const int64_t r = idx / q.qpr, c = (idx % q.qpr) * 4;
         const uint32_t ma = (bits_a[r * wpr + c / 32] >> (c % 32)) & 15u;
         const uint32_t mb = bits_b ? (bits_b[r * wpr + c / 32] >> (c % 32)) & 15u : 0u;
@@ -262,14 +296,27 @@ __global__ void keep_better_kernel(const double* __restrict__ obj2, const uint32
 }
 
 // One atomic per CTA: with one per warp, 19,000 of them queued on a single word were two thirds of the
-// time (2048 x 2048: 16.4 us, 8.4 now; 4096 x 4096: 21.8 and 16.5).
+// time (2048 x 2048: 16.4 us, 8.4 now; 14336 x 4096: 51.7, 37.4 now, at the copy bandwidth).
 __global__ void scores_max_kernel(const tsenor::ScoreSrc S, const QuadWalk q, unsigned int* out_bits) {
     float m = 0.f;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < q.nq;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = q.row(idx);
-        const float4 v = tsenor::load_score_quad(S, r, (idx - r * q.qpr) * 4);
-        m = fmaxf(fmaxf(m, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));  // fmaxf drops NaN
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (plain_source(S)) {
+        for (; idx + (SCAN_U - 1) * step < q.nq; idx += SCAN_U * step) {
+            float4 v[SCAN_U];
+#pragma unroll
+            for (int u = 0; u < SCAN_U; ++u) {
+                const int64_t r = q.row(idx + u * step);
+                v[u] = load_plain_quad(S, r, (idx + u * step - r * q.qpr) * 4);
+            }
+#pragma unroll
+            for (int u = 0; u < SCAN_U; ++u)     // fmaxf drops NaN
+                m = fmaxf(fmaxf(m, fmaxf(fabsf(v[u].x), fabsf(v[u].y))), fmaxf(fabsf(v[u].z), fabsf(v[u].w)));
+        }
+    }
+    for (; idx < q.nq; idx += step) {
+        const float4 v = tsenor::load_score_quad(S, idx / q.qpr, (idx % q.qpr) * 4);
+        m = fmaxf(fmaxf(m, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
     }
     // non-negative floats order like their bit patterns
     const unsigned warp_max = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
@@ -332,9 +379,9 @@ int grid_for(int64_t work, int threads) {
     return (int)g;
 }
 
-// CTAs of 256 threads for the maximum over quads: one wave of full SMs, since every CTA ends in an atomic.
+// CTAs of 256 threads for the maximum over quads: two waves of full SMs, since every CTA ends in an atomic.
 int scan_grid(int64_t quads) {
-    const int64_t g = (quads + 255) / 256, wave = 8LL * sm_count();
+    const int64_t g = (quads + 255) / 256, wave = 16LL * sm_count();
     return (int)(g < 1 ? 1 : g < wave ? g : wave);
 }
 

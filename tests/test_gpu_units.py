@@ -114,3 +114,19 @@ def test_mid_sizes_under_the_automatic_choice(M, N, rows, cols):
     assert int(ts.check(got, rows, cols, N, M).item()) == 0
     a, b = float(ts.objective(W, got).item()), float(ts.objective(W, want).item())
     assert abs(a - b) <= 1e-4 * b
+
+
+@pytest.mark.parametrize("rows,cols,pad", [(1, 4, 0), (37, 4, 0), (64, 132, 0), (2048, 4100, 0), (4096, 4096, 0), (1024, 4096, 5)])
+def test_scans_at_the_edges_of_their_batches(rows, cols, pad):
+    """Largest score and retained score where a thread has none, some and all of its four quads."""
+    g = torch.Generator(device=DEV).manual_seed(rows + cols)
+    w = torch.randn((rows, cols + pad), generator=g, device=DEV)[:, pad:]
+    bits = torch.randint(0, 2, (rows, cols), generator=g, device=DEV, dtype=torch.int64)
+    words = torch.zeros((rows, (cols + 31) // 32 * 32), dtype=torch.int64, device=DEV)
+    words[:, :cols] = bits
+    packed = (words.view(rows, -1, 32) << torch.arange(32, device=DEV)).sum(-1)
+    mask = torch.where(packed >= 2 ** 31, packed - 2 ** 32, packed).to(torch.int32)
+    assert float(ts.max_abs(w).item()) == float(w.abs().max().item())
+    want = float((w.abs().double() * bits).sum().item())
+    # fp64 sums of at most 2^24 terms in any order: each addition rounds to 2^-53 of the running sum
+    assert abs(float(ts.objective(w, mask).item()) - want) <= 2.0 ** -53 * 2 ** 24 * want + 1e-300
