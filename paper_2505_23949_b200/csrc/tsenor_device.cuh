@@ -1150,6 +1150,8 @@ __device__ __forceinline__ void store_plan(const Params& P, const UnitMap<G::M>&
 // warp several blocks to round): 512 x 512 4:8 43.5 -> 37.8 us, 512 x 512 8:16 53.9 -> 46.1 us,
 // 256 x 264 2:4 31.9 -> 27.5 us.
 // ---------------------------------------------------------------------------
+// A buffer is written again only after a barrier that follows its reads: in an iteration the other
+// exchange's.
 template <int M> __device__ __forceinline__ void exchange(float* buf, int lane, float mine, float2 (&all)[M / 2]) {
     buf[lane] = mine;
     __syncwarp();
@@ -1266,6 +1268,7 @@ __device__ __forceinline__ int twin_plan(const Params& P, const float* panel, fl
 #pragma unroll 1
     while (it < iters) {
         const float F = add_potential(fpot, r), Gc = add_potential(gpot, pc);
+        __syncwarp();                            // every lane has read the exchange before
         exchange<M>(ex, lane, F, x);
         exchange<M>(ex + 32, lane, Gc, y);
 #pragma unroll
@@ -1300,6 +1303,7 @@ __device__ __forceinline__ int twin_plan(const Params& P, const float* panel, fl
     }
     // final potentials, t = t0 + F + G and x = min(t, 0)
     const float F = add_potential(fpot, r), Gc = add_potential(gpot, pc);
+    __syncwarp();                                // every lane has read the exchange before
     exchange<M>(ex + 32, lane, Gc, y);           // (its barrier: no column of t0 is read any more)
 #pragma unroll
     for (int j = 0; j < M; ++j) row[j] = fminf((row[j] + F) + ((j % 2) ? y[j / 2].y : y[j / 2].x), 0.0f);
