@@ -128,15 +128,14 @@ int launch_layout(const tsenor::Params& P, cudaStream_t st) {
 //           the latency layout: w <= 6 + 600 / T, at most 16.  Latency / throughput at T = 300: w 7.8 28.7 / 30.5
 //           [27.9 / 27.8], 10.6 32.5 / 30.4; T = 100: 10.6 13.8 / 16.7, 13.8 16.2 / 16.5 [14.6 / 12.0]; T = 50: 13.8 10.5 /
 //           13.2 [8.7 / 7.6]; T = 20: 13.8 7.1 / 11.0 [5.1 / 5.1], 21.6 [6.4 / 6.1]; T = 0: 13.8 4.5 / 8.8.
-//   M = 8   latency up to three warps per scheduler (T = 300: w 10.8 48.2 / 49.7, 13.1 60.7 / 49.3); beyond, spread
-//           while w T <= 3000 and w <= 32.  Spread / throughput at T = 300: 13.1 50.3 / 49.3; T = 100: 27.7 32.9 / 37.6
-//           [29.0 / 28.5], 43 48.2 / 49.2 [42.4 / 38.8]; T = 20: 27.7 15.0 / 22.6 [9.3 / 10.8], 62 28.8 / 33.0 [17.7 / 16.6].
-//   M = 16  latency while a scheduler has one warp (T = 300: w 3.5 46.0, spread 53; 4.4 63.2, spread 58.4); beyond,
-//           spread while T <= 50 or w T <= 1800, and for 8 < w <= 12; then the build of the throughput layout with
-//           the shorter chain (V = 2) as long as all its warps are resident.  Spread / V = 2 at T = 300: 5.4 58.6 / 59.7
-//           [55.2 / 53.8], 7.8 59.4 / 60.1 [55.6 / 54.3], 10.6 68.0 / 78.2 [63.9 / 74.6], 13.8 81.9 / 79.4 [77.5 / 74.9]; T = 100:
-//           13.8 36.6 / 40.3 [30.0 / 30.7], 22 50.7 / 53.1 [41.9 / 41.3]; T = 50: 221 250 / 292 [180 / 180]; T = 20: 221 191 /
-//           227 [94 / 104].  V = 2 / throughput at T = 300: 13.8 79.4 / 87.6, 31 142.3 / 143.9.
+//   M = 8   latency up to three warps per scheduler; beyond, spread while w <= 32 and w T <= 3200, or w <= 28 and
+//           w T <= 6400.  Spread / throughput, Gaussian (Student-t in brackets): T = 300: 13.1 51.2 / 53.5 [34.8 / 47.6], 18.3 58.1 /
+//           75.1 [46.5 / 66.0], 21.2 67.5 / 75.4 [49.3 / 55.6], 24.3 78.6 / 75.2 [51.3 / 62.4]; T = 200: 27.7 55.6 / 56.3, 31.2 63.4 / 56.6;
+//           T = 100: 31.2 37.5 / 38.3, 43 50.2 / 50.2; T = 20: 27.7 15.4 / 23.2, 62 28.8 / 33.0 [Algorithm 1 alone 17.7 / 16.6].
+//   M = 16  latency while a scheduler has one warp (T = 300: w 3.5 44.6, spread 53; 4.4 63.2, spread 57.5); beyond,
+//           spread while T <= 50, w T <= 1800 or w <= 16.  Spread / throughput at T = 300: 15.6 80.9 [Student-t 42.3] / 92,
+//           17.5 - / 108.7 [51.4]; T = 100: 22 50.7 / 53.1 [Algorithm 1 alone 41.9 / 41.3]; T = 50: 221 250 / 292 [180 / 180];
+//           T = 20: 221 191 / 227 [94 / 104].
 //   M = 32  the same layout in both builds: the one for latency while all its warps are resident (6.9 86.1 /
 //           93.0; 15.6 142.9 / 145.1).
 // The stopping test does not say beforehand how many iterations it will run: spread up to w = 16 (768 x 768
@@ -150,8 +149,8 @@ template <int M, bool EE> bool spread_is_best(int64_t warps, int64_t sms, int T)
     const auto up_to = [&](int64_t w) { return warps <= w * sms; };
     const int64_t wT = warps * T;
     if (EE && up_to(16)) return true;
-    if (M == 8) return up_to(32) && wT <= 3000 * sms;
-    return T <= 50 || wT <= 1800 * sms || (up_to(12) && !up_to(8));
+    if (M == 8) return (up_to(32) && wT <= 3200 * sms) || (up_to(28) && wT <= 6400 * sms);
+    return T <= 50 || wT <= 1800 * sms || up_to(16);
 }
 // Rounding alone has no iterations to share lanes for, and units of one mask word are one rounding pass: more
 // warps and nothing serial (log-plans, us against the wider units: 1024 x 1024 M = 8 7.0 / 10.1, M = 16 9.3 / 12.1;
@@ -175,9 +174,6 @@ int launch(const tsenor::Params& P, cudaStream_t st) {
         if constexpr (M == 8 || M == 16)
             if (policy == TSENOR_LAYOUT_AUTO && spread_is_best<M, EE>(warps, sms, P.iters))
                 return launch_layout<M, MODE, 3, EE>(P, st);
-        if constexpr (M == 16 && !EE)
-            if (policy == TSENOR_LAYOUT_AUTO && unit_count<M, 2>(P, &nbp) <= 16 * sms)
-                return launch_layout<M, MODE, 2, EE>(P, st);
         return launch_layout<M, MODE, 0, EE>(P, st);
     }
 }

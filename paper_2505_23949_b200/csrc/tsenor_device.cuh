@@ -60,7 +60,6 @@ __device__ __forceinline__ int bounds_end() { return 0; }
 //          shared-memory broadcasts an iteration where sub-tiles need six to eight dependent
 //          shuffles.  M = 32: the sub-tiles of V = 0 with what a lone warp waits for taken out: scalar
 //          adds in the exchanges, one vote on the range test, scores kept beside the keys.
-//   V = 2  M = 16 in between: the sub-tiles of V = 0, the same taken out.
 //   V = 3  spread, M = 8 and 16: a block over M lanes as in V = 1 (so a unit rounds in one pass), but
 //          in sub-tiles, each element once: for what lies between V = 1 and a full GPU, and for few iterations.
 // ---------------------------------------------------------------------------
@@ -175,9 +174,17 @@ __device__ __forceinline__ void all_gather(float (&v)[K], int base) {
 // Adds log2 of a running product of scalings (sign -1: of its reciprocal) to a Kahan-compensated potential.  The potentials
 // (one row and one column at M = 32) live in shared memory, private to the lane: they are touched
 // once in up to 48 iterations, and without them the loop fits in the 96 registers of 20 warps per SM.
+// Near 1, where the products of converged blocks are, by the Taylor series of log2(1 + t) (error below 4e-10;
+// lg2.approx is only good to 2^-22 there, and what comes in at the end stays in the plan).
+__device__ __forceinline__ float log2_of_product(float p) {
+    const float t = p - 1.0f;
+    const float series = t * fmaf(t, fmaf(t, fmaf(t, -0.36067376f, 0.48089835f), -0.72134752f), 1.44269504f);
+    return fabsf(t) < 0.015625f ? series : lg2_approx(p);
+}
+template <bool LAST = false>
 __device__ __forceinline__ float add_potential(float2* p, float prod, float sign = 1.0f) {
     const float2 c = *p;                     // value, compensation
-    const float y = sign * lg2_approx(prod) - c.y;
+    const float y = sign * (LAST ? log2_of_product(prod) : lg2_approx(prod)) - c.y;
     const float v = c.x + y;
     *p = make_float2(v, (v - c.x) - y);
     return v;
@@ -226,7 +233,7 @@ __device__ __forceinline__ float add_potential(float2* p, float prod, float sign
 // float2 of it for the owned potentials.
 // ---------------------------------------------------------------------------
 constexpr int CHECK = 4;     // iterations between range tests of the accumulated scalings
-constexpr int MAXRUN = 48;   // longest run of linear-domain iterations (multiple of CHECK)
+constexpr int MAXRUN = 48;   // longest run of linear-domain iterations (multiple of CHECK; see run_length)
 
 // Exponent field outside [127-16, 127+16] <=> product outside [2^-16, 2^17).  A product that is inf or
 // NaN (exponent field 255: a block poisoned by a non-finite score) does not vote, so that it cannot
@@ -246,10 +253,10 @@ __device__ __forceinline__ unsigned window_distance(float p) { return __float_as
 // hold V = U / R_i with R_i the product of the rho_i since the last rebuild, and
 // one multiply per element (by kap_j) is left.  Four fp32 operations per element
 // and iteration, in one of two forms:
-//   M >= 16  rs[a] = R_i:    e = sat(V R_i) = min(U, 1) by a saturating multiply (FMA pipe), row
+//   M = 32   rs[a] = R_i:    e = sat(V R_i) = min(U, 1) by a saturating multiply (FMA pipe), row
 //            sums of e give rho_i = N / sum, column sums are sum_i e_ij rho_i, kap_j = N / sum,
 //            R_i <- R_i rho_i in every lane of the row;
-//   M <= 8   rs[a] = 1/R_i:  m = min(V, 1/R_i) = e / R_i (the clip threshold moves instead of the
+//   M <= 16  rs[a] = 1/R_i:  m = min(V, 1/R_i) = e / R_i (the clip threshold moves instead of the
 //            tile), whose row sums s give the new 1/R_i = s / N and the column sums c = sum_i m_ij / s_i
 //            (= sum_i e_ij rho_i / N) give kap_j = 1 / c.  Only s carries a rounding from one iteration
 //            to the next: 1/N is split in two floats, so that s / N is rounded once whatever N is.
@@ -258,8 +265,10 @@ __device__ __forceinline__ unsigned window_distance(float p) { return __float_as
 // eighteen matrices) 1.36e-7 at 1:4 by products and 1.14e-7 by thresholds, 3.15e-7 and 2.84e-7 at 3:4,
 // 7.1e-7 and 6.3e-7 at 7:8; of the plan 3.8e-7 and 3.3e-7 at 1:4.  Time 946 us against 930 (4096 x 4096
 // 2:4), 858 against 853 (4:8): no factor N is left, which pays for the half-rate min.  (Without the split of
-// 1/N 912 and 831, but at N = 3, 6, 7 no more exact than the products.)  At M >= 16 the thresholds need a
-// second gather.
+// 1/N 912 and 831, but at N = 3, 6, 7 no more exact than the products.)  At M = 16, where the thresholds need a
+// second gather, the two take the same time (875 us, 4096 x 4096 8:16), but by thresholds a converged block
+// recurs sooner (see below; Student-t scores 301 us against 409) and the log-plan is as exact or more so (15:16:
+// 0.73 of the distance).  At M = 32 the thresholds are 3.5 % slower.
 //
 // Whether the exchanges' adds and (M >= 16) the row factors are packed too (PACK) is a matter of how the
 // packed and the scalar instructions of the other warps interleave on the FMA pipes: the factors
@@ -267,7 +276,7 @@ __device__ __forceinline__ unsigned window_distance(float p) { return __float_as
 // the stopping test's mixture, only see the packed ones' longer latency (14336 x 32: 69.4 us
 // without, 74.5 with).
 template <int M> struct PackAdd { static constexpr bool value = (M >= 16); };
-template <int M> struct ByThreshold { static constexpr bool value = (M <= 8); };
+template <int M> struct ByThreshold { static constexpr bool value = (M <= 16); };
 
 // 1/N as the sum of two floats (made on the host).
 struct InvN {
@@ -278,11 +287,47 @@ struct InvN {
     }
 };
 
+// Copy of a lane's state in local memory (registers are what the loop is short of).
+template <int CELLS> struct Snapshot {
+    alignas(8) unsigned cell[CELLS];
+    __device__ __forceinline__ unsigned* hidden() {     // keeps the compiler from making registers of it
+        unsigned* p = cell;
+        asm volatile("" : "+l"(p));
+        return p;
+    }
+    template <int K> __device__ __forceinline__ void take(int at, const float (&v)[K]) {
+        unsigned* const p = hidden() + at;
+#pragma unroll
+        for (int k = 0; k < K; ++k) p[k] = __float_as_uint(v[k]);
+    }
+    template <int K> __device__ __forceinline__ void take(int at, const float2 (&v)[K]) {
+        uint2* const p = reinterpret_cast<uint2*>(hidden() + at);
+#pragma unroll
+        for (int k = 0; k < K; ++k) p[k] = make_uint2(__float_as_uint(v[k].x), __float_as_uint(v[k].y));
+    }
+    // Bits in which v differs from what was taken.
+    template <int K> __device__ __forceinline__ unsigned differ(int at, const float (&v)[K]) {
+        const unsigned* const p = hidden() + at;
+        unsigned d = 0u;
+#pragma unroll
+        for (int k = 0; k < K; ++k) d |= p[k] ^ __float_as_uint(v[k]);
+        return d;
+    }
+    template <int K> __device__ __forceinline__ unsigned differ(int at, const float2 (&v)[K]) {
+        const uint2* const p = reinterpret_cast<const uint2*>(hidden() + at);
+        unsigned d = 0u;
+#pragma unroll
+        for (int k = 0; k < K; ++k) d |= (p[k].x ^ __float_as_uint(v[k].x)) | (p[k].y ^ __float_as_uint(v[k].y));
+        return d;
+    }
+};
+
+// KEEP: last receives the column scalings of the lines this lane owns.
 // DELTA: also returns this lane's share of the marginal violation seen by the iteration,
 // max over the lines it owns of |row sum of e - N| and |column sum of e rho - N|.
-template <class G, bool PACK, bool DELTA = false>
+template <class G, bool PACK, bool DELTA = false, bool KEEP = false>
 __device__ __forceinline__ float dykstra_step(float2 (&V)[G::T::MR][G::T::MC / 2], float (&rs)[G::T::MR],
-                                              float (&Pc)[G::CO], float Nf, const InvN& iN) {
+                                              float (&Pc)[G::CO], float (&last)[G::CO], float Nf, const InvN& iN) {
     using T = typename G::T;
     constexpr int M = G::M;
     constexpr bool THR = ByThreshold<M>::value;
@@ -328,6 +373,7 @@ __device__ __forceinline__ float dykstra_step(float2 (&V)[G::T::MR][G::T::MC / 2
     for (int k = 0; k < CO; ++k) {
         kap[k] = THR ? rcp_approx(cp[k]) : Nf * rcp_approx(cp[k]);
         Pc[k] *= kap[k];
+        if (KEEP) last[k] = kap[k];
     }
     all_gather<MC, PR>(kap, PC);
     if constexpr (THR) {
@@ -363,6 +409,39 @@ __device__ __forceinline__ float dykstra_step(float2 (&V)[G::T::MR][G::T::MC / 2
 // Returns the number of iterations run: iters, or fewer in the stopping-test mode (EE, ee_eps > 0):
 // after every group of CHECK iterations, i.e. at iterations 5, 9, 13, ... of Algorithm 1, the
 // warp stops once the marginal violation of every block it holds is below ee_eps.
+// ---------------------------------------------------------------------------
+// Recurring states.  Algorithm 1 converges, and the state of the linear-domain loop (V and the row
+// factors) is a few thousand floats that depend on nothing but themselves: once the scalings are within
+// rounding of 1 it returns, bit for bit, to where it was one, two or four iterations before.  All that
+// is left of the T iterations then repeats what was seen, so the warp runs (T - t) mod 4 more and is done:
+// its state is the one that all T would end in.  Nothing is assumed about convergence; a state that has not
+// recurred, in every bit and in every block of the warp, is iterated on.
+//
+// Looking costs a copy of the state and a comparison per four iterations, so a warp looks only once a run
+// has ended with every column scaling within NEAR_ONE of 1, and in a run of its own (at most LOOKS of them)
+// that begins with a rebuild: that takes out the roundings which V has gathered, so that the plan is as
+// exact as after all T (log-plan's distance from the fp64 iterate, mean over 1:M to M-1:M and four
+// distributions, against running on: 1.00 at M = 4 and 8, 0.97 at 16, 1.00 at 32).  The first runs are
+// short, since that is when most blocks of heavy-tailed scores get there: of |Student-t| and outlier-column
+// matrices under tau = 200 / max nearly all within 30 to 80 iterations; of Gaussian ones hardly any in 300.
+// 4096 x 4096, us before / now, for Student, outlier, Wanda-style and Gaussian scores:
+//   2:4    933 / 296, 928 / 438, 931 / 680, 924 / 902        4:8    862 / 315, 857 / 474, 863 / 574, 851 / 835
+//   8:16   871 / 284, 863 / 438, 872 / 633, 858 / 856        16:32  864 / 375, 855 / 418, 865 / 671, 855 / 864
+// V = 1 does not look: with a warp or two per scheduler the slowest block of the matrix sets the time
+// (256 x 264 2:4 with outlier columns: 26.2, 28.1 with looking).
+// ---------------------------------------------------------------------------
+constexpr float NEAR_ONE = 3.6e-7f;      // three units in the last place above 1
+constexpr int LOOKS = 2;
+template <class G, bool EE> struct Recurrence { static constexpr bool value = !EE && (G::V == 0 || G::V == 3); };
+// Length of the run that starts at iteration t: one more than a multiple of CHECK, so that the loop after the
+// groups of CHECK leaves the scalings to be looked at in registers.  At M = 32 one short run, else two, where
+// enough iterations are left to pay for a rebuild more (2048 x 2048 4:8, 50 iterations: 73.6 us without, 80.1 with).
+template <class G, bool LOOK> __device__ __forceinline__ int run_length(int t, int iters) {
+    if (!LOOK) return MAXRUN;
+    return (G::V == 0 && iters >= 120 && t <= (G::M == 32 ? 1 : MAXRUN / 2 + 2)) ? MAXRUN / 2 + 1 : MAXRUN + 1;
+}
+constexpr int WORTH_LOOKING = 32;        // iterations left
+
 template <class G, bool EE>
 __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], float* stash, float2* pot, int lane,
                                                float Nf, const InvN& iN, float log2N, int iters, float ee_eps) {
@@ -371,6 +450,7 @@ __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], f
     constexpr int RO = G::RO, CO = G::CO;
     constexpr int MP = MC / 2, NQ = MR * MC / 4;
     constexpr bool PACK = (G::V == 0 && !EE);
+    constexpr bool LOOK = Recurrence<G, EE>::value;
     float F[MR], Gc[MC];
     float rs[MR];
     float Pc[CO];              // products of kap since the last rebuild; rs[0 .. RO): those of rho, or 1 / them
@@ -430,7 +510,9 @@ __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], f
     // Iterations 1 .. iters-1 in runs: rebuild U from the potentials, then groups of
     // CHECK iterations with the range test of the accumulated scalings between groups.
     float2 V[MR][MP];
+    float last[CO];            // column scalings of the last iteration
     int it = 1;
+    int look = 0;              // 2 x (runs that looked for a recurring state) + (the next one is to)
 #pragma unroll 1
     while (it < iters) {
 #pragma unroll
@@ -452,24 +534,8 @@ __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], f
         }
 #pragma unroll
         for (int a = 0; a < MR; ++a) rs[a] = 1.0f;     // R_i = 1
-        const int run_end = (iters - it > MAXRUN) ? it + MAXRUN : iters;
-        bool wide = false;
-#pragma unroll 1
-        while (!wide && it + CHECK <= run_end) {
-#pragma unroll(EE && G::M == 32 ? 1 : CHECK)   // (the stopping test at M = 32 is mostly code that runs once)
-            for (int u = 0; u < CHECK - 1; ++u) dykstra_step<G, PACK>(V, rs, Pc, Nf, iN);
-            if constexpr (EE) {
-                const float delta = dykstra_step<G, PACK, true>(V, rs, Pc, Nf, iN);
-                if (__all_sync(FULL, delta < ee_eps)) {   // every block of the warp has converged
-                    it += CHECK;
-                    iters = it;
-                    wide = true;                          // skips the remainder loop as well
-                    break;
-                }
-            } else {
-                dykstra_step<G, PACK>(V, rs, Pc, Nf, iN);
-            }
-            it += CHECK;
+        int run_end = LOOK ? min(iters, it + run_length<G, LOOK>(it, iters)) : (iters - it > MAXRUN) ? it + MAXRUN : iters;
+        const auto out_of_range = [&]() {
             // V = 0: a first, cheap test (a subtraction and a maximum per line, every four iterations)
             // that also catches inf, NaN and zero; what it catches is looked at properly (1.5 to 4 %
             // of the loop).  A lone warp waits longer for the second vote than it saves.
@@ -478,25 +544,81 @@ __device__ __forceinline__ int dykstra_iterate(float (&t)[G::T::MR][G::T::MC], f
             for (int k = 0; k < RO; ++k) far = max(far, window_distance(rs[k]));
 #pragma unroll
             for (int k = 0; k < CO; ++k) far = max(far, window_distance(Pc[k]));
+            bool w = false;
             if (G::V != 0 || __any_sync(FULL, far > WINDOW)) {
-                bool w = false;
 #pragma unroll
                 for (int k = 0; k < RO; ++k) w |= out_of_window(rs[k]);
 #pragma unroll
                 for (int k = 0; k < CO; ++k) w |= out_of_window(Pc[k]);
-                wide = __any_sync(FULL, w);
+                w = __any_sync(FULL, w);
             }
-        }
-        if (!wide) {   // fewer than CHECK iterations left (end of the last run only)
+            return w;
+        };
+        bool wide = false;
+        if (LOOK && (look & 1)) {
+            Snapshot<MR * MC + MR> before;
+            bool recurs = false;
 #pragma unroll 1
-            for (; it < run_end; ++it) dykstra_step<G, PACK>(V, rs, Pc, Nf, iN);
+            while (!wide && !recurs && it + CHECK <= run_end) {
+#pragma unroll
+                for (int a = 0; a < MR; ++a) before.take(a * MC, V[a]);
+                before.take(MR * MC, rs);
+#pragma unroll 1
+                for (int u = 0; u < CHECK; ++u) dykstra_step<G, PACK>(V, rs, Pc, last, Nf, iN);
+                it += CHECK;
+                unsigned differ = before.differ(MR * MC, rs);
+#pragma unroll
+                for (int a = 0; a < MR; ++a) differ |= before.differ(a * MC, V[a]);
+                wide = out_of_range();
+                recurs = !wide && __all_sync(FULL, differ == 0u);
+            }
+            if (recurs) run_end = it + (iters - it) % CHECK;
+            if (!wide) {
+#pragma unroll 1
+                for (; it < run_end; ++it) dykstra_step<G, PACK>(V, rs, Pc, last, Nf, iN);
+            }
+            if (recurs) break;
+            look += 2;
+            if (wide || look > 2 * LOOKS || iters - it < WORTH_LOOKING) look &= ~1;
+            continue;
+        }
+#pragma unroll 1
+        while (!wide && it + CHECK <= run_end) {
+            // Two iterations of code where many warps share the instruction cache with other warps' rounding
+            // (four: 5 to 15 % slower on matrices that converge), four where few do (two: 4 % slower) or an iteration
+            // is short (65536 x 4 2:4: 30.8 us, 33.0 with two).  The stopping test at M = 32 is mostly code that runs once.
+#pragma unroll(EE && G::M == 32 ? 1 : (EE || G::V != 0 || G::M == 4) ? CHECK : 2)
+            for (int u = 0; u < CHECK - (EE ? 1 : 0); ++u) dykstra_step<G, PACK>(V, rs, Pc, last, Nf, iN);
+            if constexpr (EE) {
+                const float delta = dykstra_step<G, PACK, true>(V, rs, Pc, last, Nf, iN);
+                if (__all_sync(FULL, delta < ee_eps)) {   // every block of the warp has converged
+                    it += CHECK;
+                    iters = it;
+                    wide = true;                          // skips the remainder loop as well
+                    break;
+                }
+            }
+            it += CHECK;
+            wide = out_of_range();
+        }
+        if (!wide) {   // fewer than CHECK iterations left
+#pragma unroll
+            for (int k = 0; k < CO; ++k) last[k] = 2.0f;  // (no value of the loop above has to be kept)
+#pragma unroll 1
+            for (; it < run_end; ++it) dykstra_step<G, PACK, false, LOOK>(V, rs, Pc, last, Nf, iN);
+            if constexpr (LOOK) {
+                float off = 0.0f;                         // (fmaxf drops NaN)
+#pragma unroll
+                for (int k = 0; k < CO; ++k) off = fmaxf(off, fabsf(last[k] - 1.0f));
+                if (look < 2 * LOOKS && iters - it >= WORTH_LOOKING && __all_sync(FULL, off <= NEAR_ONE)) look |= 1;
+            }
         }
     }
     // final potentials and t = t0 + F + G
 #pragma unroll
-    for (int k = 0; k < RO; ++k) F[k] = add_potential(fpot + k * 32, rs[k], SIGN);
+    for (int k = 0; k < RO; ++k) F[k] = add_potential<true>(fpot + k * 32, rs[k], SIGN);
 #pragma unroll
-    for (int k = 0; k < CO; ++k) Gc[k] = add_potential(gpot + k * 32, Pc[k]);
+    for (int k = 0; k < CO; ++k) Gc[k] = add_potential<true>(gpot + k * 32, Pc[k]);
     all_gather<MR, PC>(F, 1);
     all_gather<MC, PR>(Gc, PC);
 #pragma unroll
@@ -1276,9 +1398,9 @@ __device__ __forceinline__ void store_plan(const Params& P, const UnitMap<G::M>&
 // of the linear iterate (Vr) and, a second time, column i (Vc) with the factors of all rows (Ra); both
 // copies see the same operations and stay equal bit for bit.  A row sum and a column sum are then a
 // lane's own, and an iteration is two exchanges long: rho to the lanes of the block (one store, M / 4
-// broadcast loads of 16 bytes), kap likewise (M <= 8: 1 / s and kap, and the new thresholds beside 1 / s).  What bounds it is that chain: sum, reciprocal,
+// broadcast loads of 16 bytes), kap likewise (here 1 / s and kap, and the new thresholds beside 1 / s).  What bounds it is that chain: sum, reciprocal,
 // exchange, sum, reciprocal, exchange.  The stash of t0 is the M x 32 matrix in `k` itself, read by
-// rows and by columns.  pot: 64 float2 for the owned potentials, then 64 floats (M <= 8: 96) for the exchange.
+// rows and by columns.  pot: 64 float2 for the owned potentials, then 96 floats for the exchange.
 // The numbers are those of dykstra_iterate, whose comments apply; only the order of the sums differs.
 // A lone warp takes 143 / 168 / 225 clocks an iteration for M = 4 / 8 / 16, where a block spread over M
 // lanes in sub-tiles took 181 / 229 / 267 and the throughput layout takes 134 / 210 / 244 (but leaves one
@@ -1453,7 +1575,7 @@ __device__ __forceinline__ int twin_plan(const Params& P, const float* panel, fl
         }
     }
     // final potentials, t = t0 + F + G and x = min(t, 0)
-    const float F = add_potential(fpot, r, SIGN), Gc = add_potential(gpot, pc);
+    const float F = add_potential<true>(fpot, r, SIGN), Gc = add_potential<true>(gpot, pc);
     __syncwarp();                                // every lane has read the exchange before
     exchange<M>(ex + 32, lane, Gc, y);           // (its barrier: no column of t0 is read any more)
 #pragma unroll
@@ -1484,12 +1606,12 @@ template <class G, int MODE, bool EE> struct SmemLayout {   // of one warp
 template <int M, int V, bool EE> struct MinWarps {
     static constexpr int value = (V == 1) ? 12 : (M >= 16 && V == 0 && !EE) ? 20 : 16;
 };
-// Warps per CTA.  One: 3 to 25 % faster than four on ragged widths (finer tail) and never slower,
-// with one exception.  The stopping test at M = 32 runs through the kernel's whole code for a dozen
-// iterations of work; four warps that go through it together (barriers after the loader and before
-// the rounding stage) share what they fetch of it (14336 x 4096, Student scores: 663 us apart, 606 together;
-// Gaussian ones, which run all 300 iterations, 3.00 ms apart, 3.07 together).
-template <int M, int V, bool EE> struct CtaWarps { static constexpr int value = (M == 32 && V == 0 && EE) ? 4 : 1; };
+// Warps per CTA.  One: 3 to 25 % faster than four on ragged widths (finer tail), except where much of the
+// time goes into code that runs once, as at M = 32 with blocks that converge early: four warps that go
+// through it together (barriers after the loader and before the rounding stage) share what they fetch of it
+// (14336 x 4096, Student scores: 1,420 us apart, 1,310 together; Gaussian ones 2.95 ms both ways; two warps
+// 1,415, five 1,290 and 3.02.  Stopping test: 663 and 606 us; Gaussian 3.00 and 3.07 ms).
+template <int M, int V, bool EE> struct CtaWarps { static constexpr int value = (M == 32 && V == 0) ? 4 : 1; };
 
 // Cells of a lane's sub-tile in a shared-memory panel.
 template <class G> struct SubTile {
