@@ -601,6 +601,9 @@ def run_cuda(args, rank, world, local_rank):
                 "bound": "alu", "pipe": "fp32 dispatch (add/mul/fma/min), 4 lane-ops per element and iteration",
                 "achieved": achieved / 1e12, "peak": fp32_peak / 1e12, "unit": "Tlaneop/s",
                 "frac": achieved / fp32_peak,
+                "frac_note": "operations of all T iterations over the time and the peak: work delivered. Blocks whose "
+                             "state recurs bit for bit are not iterated further, so it can exceed 1 on matrices that "
+                             "converge; pipe utilisation is in the profile summary",
                 # time a kernel doing the scope table's per-unit fp32 work (9 M^2 T, its one-exp model;
                 # 12 M^2 T for the paper's listing) would need at that peak, over the measured time
                 "vs_fp32_bound_one_exp_model": achieved * 9 / 4 / fp32_peak,

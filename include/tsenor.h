@@ -177,8 +177,10 @@ typedef struct tsenor_scores {
                             a warp holds one block).  0: fixed iteration count (the
                             parity contract).                                          */
     uint64_t *dev_iters_out; /* optional, with or without early_exit_eps: *dev_iters_out
-                            (device, zeroed by the caller) += iterations run, summed over
-                            all blocks                                                 */
+                            (device, zeroed by the caller) += number of the iteration whose
+                            plan a block ended with (`iters` without early_exit_eps, also
+                            where the last ones repeat earlier ones bit for bit and are not
+                            run), summed over all blocks                               */
 } tsenor_scores_t;
 
 /* tsenor_solve on the score matrix described by *s (same arguments otherwise). */
