@@ -36,8 +36,9 @@ NOMINAL_SM_MHZ = 1965.0
 # summarised in PROFILE_SUMMARY (not measured by this script: they go stale if the kernel changes
 # and the capture is not repeated, which is why the JSON line names their source).
 PROFILE_SUMMARY = "profiles/tsenor_kernel_all_sizes_current.md"
-NCU_DRAM_BYTES_PER_LAUNCH = 244.17e6      # dram__bytes_read.sum + dram__bytes_write.sum
-NCU_WARP_INST_PER_BLOCK_ITER = 135.4      # smsp__inst_executed.sum / (57,344 blocks x 300 iterations)
+NCU_DRAM_BYTES_PER_LAUNCH = 243.29e6      # dram__bytes_read.sum + dram__bytes_write.sum
+NCU_WARP_INST_PER_BLOCK_ITER = 134.1      # smsp__inst_executed.sum / (16,384 blocks x 300 iterations), 4096x4096
+                                          # Gaussian scores, which run all of the iterations
 
 
 def fp32_lane_ops_per_block(M, T):
