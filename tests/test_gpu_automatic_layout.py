@@ -16,8 +16,8 @@ CASES = [
     (4, 2, 512, 516, 20), (4, 1, 384, 388, 300), (4, 3, 520, 516, 100),           # latency, latency, throughput
     (8, 4, 640, 648, 60), (8, 3, 768, 776, 60), (8, 5, 776, 768, 300),            # latency, spread, throughput
     (16, 8, 496, 528, 60), (16, 5, 640, 656, 60), (16, 8, 880, 912, 300),         # latency, spread, spread
-    (16, 8, 1024, 1024, 300), (16, 11, 1040, 1008, 300), (16, 9, 768, 784, 300),  # the mid-size build
-    (16, 8, 16 * 7104, 16, 60), (8, 2, 8 * 9000, 8, 60),                          # slabs: mid-size build, spread
+    (16, 8, 1024, 1024, 300), (16, 11, 1040, 1008, 300), (16, 9, 768, 784, 300),  # spread
+    (16, 8, 16 * 7104, 16, 60), (8, 2, 8 * 9000, 8, 60),                          # slabs: spread, spread
     (32, 16, 1280, 1248, 60),                                                     # latency
 ]
 

@@ -66,7 +66,7 @@ def test_no_index_check_fires_and_results_equal_the_normal_build(checked_library
         assert np.array_equal(g, w)
 
 
-# sizes whose builds only the automatic choice reaches: spread (M = 8, 16) and the mid-size build of M = 16
+# sizes whose builds only the automatic choice reaches: spread (M = 8, 16)
 @pytest.mark.parametrize("M,N,rows,cols", [(8, 3, 768, 776), (16, 5, 640, 656), (16, 8, 1040, 1008)])
 def test_no_index_check_fires_under_the_automatic_choice(checked_library, M, N, rows, cols):
     iters = 60 if rows < 1000 else 300
